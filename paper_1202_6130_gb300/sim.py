@@ -13,12 +13,16 @@ from . import _lib as L
 
 
 class TorchAllocator:
-    """lbm_allocator backed by torch's caching allocator on one device."""
+    """lbm_allocator backed by torch's caching allocator on one device.  Blocks
+    come from the pool of ``stream``, the stream the owner's work runs on: a
+    block that another stream's tensors gave back may still be written by
+    kernels pending there, and the owner's stream does not wait for those."""
 
-    def __init__(self, device):
+    def __init__(self, device, stream=None):
         import torch
         self.torch = torch
         self.device = torch.device(device)
+        self.stream = stream if isinstance(stream, torch.cuda.Stream) else None
         self.live = {}
         self._alloc = L.ALLOC_FN(self._alloc_cb)
         self._free = L.FREE_FN(self._free_cb)
@@ -26,7 +30,8 @@ class TorchAllocator:
 
     def _alloc_cb(self, nbytes, user):
         try:
-            t = self.torch.empty(int(nbytes), dtype=self.torch.uint8, device=self.device)
+            with self.torch.cuda.stream(self.stream):  # None: the current stream
+                t = self.torch.empty(int(nbytes), dtype=self.torch.uint8, device=self.device)
         except Exception:  # out of memory -> NULL -> LBM_ENOMEM
             return None
         p = t.data_ptr()
@@ -76,7 +81,7 @@ class Simulation:
         self.nx, self.ny, self.Q = int(nx), int(ny), int(lattice)
         self.device = torch.device("cuda", torch.cuda.current_device())
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
-        self.allocator = TorchAllocator(self.device) if use_torch_allocator else None
+        self.allocator = TorchAllocator(self.device, self.stream) if use_torch_allocator else None
         ctx = ctypes.c_void_p()
         rc = self.lib.lbm_create(ctypes.byref(p),
                                  ctypes.byref(self.allocator.struct) if self.allocator else None,
@@ -258,7 +263,7 @@ class Batch:
         self.lib = L.load()
         dev = torch.device("cuda", torch.cuda.current_device()) if device is None else device
         self.stream = stream if stream is not None else torch.cuda.Stream(dev)
-        self.allocator = TorchAllocator(dev) if use_torch_allocator else None
+        self.allocator = TorchAllocator(dev, self.stream) if use_torch_allocator else None
         h = ctypes.c_void_p()
         L.check_batch(self.lib.lbm_batch_create(
             ctypes.byref(self.allocator.struct) if self.allocator else None,

@@ -231,3 +231,19 @@ def test_many_members_span_several_launch_chunks(pkg, storage):
     for s, r in zip(sims[:5], ref):
         np.testing.assert_array_equal(s.populations(), r.populations())
     b.close()
+
+
+def test_batch_memory_comes_from_the_pool_of_the_batch_stream(pkg):
+    """The batch fills its descriptors on its own stream, which does not wait
+    for the current one: its memory must not be a block that the current
+    stream's tensors just gave back (their kernels may be pending)."""
+    import torch
+    b = pkg.Batch()
+    n = 64 << 20
+    t = torch.empty(n, dtype=torch.uint8, device="cuda")
+    freed = t.data_ptr()
+    del t
+    p = b.allocator._alloc_cb(n, None)
+    assert p != freed
+    b.allocator._free_cb(p, None)
+    b.close()
