@@ -4,8 +4,8 @@ of the HBM roofline.
 Workload: the 8192x4096 D2Q9 lattice with 64 drops (R ~ U[40, 120], seed 1) on a
 heterogeneous wall (thickness 3 + 1.5 sin(2 pi 8 x / nx)), exponential
 pseudo-potential G = -5.5, tau = 1, core 0.1 / tail 0.05 wall potential.
-A bench "step" is one LB time step over the whole lattice: one launch of the
-fused kernel.  Population buffers (2 x 1.2 GB in FP32) are far larger than L2,
+A bench "step" is one LB time step over the whole lattice; a launch of the fused
+kernel advances one or two.  Population buffers (2 x 1.2 GB in FP32) are far larger than L2,
 so no flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--storage fp32|fp16s|bf16s|fp64]
@@ -53,7 +53,7 @@ def workload_name(nx: int, ny: int, lattice: int) -> str:
     return WORKLOAD.replace("8192x4096", f"{nx}x{ny}").replace("D2Q9", f"D2Q{lattice}")
 
 
-KERNEL_SOURCES = ["step_kernel.cuh", "node.cuh", "f2.cuh", "tma.cuh", "lattice.cuh", "launch.cuh",
+KERNEL_SOURCES = ["step_kernel.cuh", "tile_kernel.cuh", "node_update.cuh", "step_args.cuh", "node.cuh", "f2.cuh", "tma.cuh", "lattice.cuh", "launch.cuh",
                   "step_impl.cuh", "engine.cu"]
 
 
@@ -378,12 +378,19 @@ PER_STORAGE = ((9, "fp16s", 400), (9, "bf16s", 400), (9, "fp64", 20),
                (21, "fp32", 100), (21, "fp16s", 150), (21, "bf16s", 150))
 
 
+def steps_per_launch(lay: dict, lattice: int, storage: str) -> int:
+    """Time steps that one launch of consecutive steps advances."""
+    return 2 * lattice * BYTES[storage] // lay["bytes_per_node"]
+
+
 def roofline_of(torch, local, lattice: int, storage: str, N: int, steps: int, t: float,
-                clocks: dict) -> dict:
-    """Roofline of the fused kernel: algorithmic bytes per node update (2 Q s)
-    against the measured HBM copy rate, or for FP64 storage the executed FP64
-    flops against the DFMA peak derived from the SM count and clock."""
+                clocks: dict, lay: dict) -> dict:
+    """Roofline of the fused kernel: algorithmic bytes per node update (2 Q s per
+    launch, over the steps that a launch advances) against the measured HBM copy
+    rate, or for FP64 storage the executed FP64 flops against the DFMA peak
+    derived from the SM count and clock."""
     traffic = ncu_traffic(storage, lattice)
+    kernel = "lbm::step_kernel" if lay["stages"] > 1 else "lbm::tile_kernel"
     if storage == "fp64":
         props = torch.cuda.get_device_properties(local)
         mhz = clocks.get("sm_max_mhz") or 2070.0
@@ -393,13 +400,14 @@ def roofline_of(torch, local, lattice: int, storage: str, N: int, steps: int, t:
                 "frac": fach / fpeak, "traffic": traffic,
                 "peak_source": f"derived: {props.multi_processor_count} SMs x "
                                f"{FP64_DFMA_PER_SM_CLK} DFMA/clk x 2 flop x {mhz:.0f} MHz",
-                "flops_per_node": FP64_FLOPS_PER_NODE[lattice], "kernel": "lbm::step_kernel"}
+                "flops_per_node": FP64_FLOPS_PER_NODE[lattice], "kernel": kernel}
     peak, peak_kind = measured_peaks()
-    b_node = 2 * lattice * BYTES[storage]
+    b_node = lay["bytes_per_node"]
     achieved = b_node * N * steps / t / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": traffic, "peak_source": f"{peak_kind} hbm_gbs",
-            "bytes_per_node": b_node, "kernel": "lbm::step_kernel"}
+            "bytes_per_node": b_node, "kernel": kernel,
+            "steps_per_launch": steps_per_launch(lay, lattice, storage)}
 
 
 def measure_per_storage(pkg, torch, W, local: int, nx: int, ny: int, variants=PER_STORAGE):
@@ -430,7 +438,7 @@ def measure_per_storage(pkg, torch, W, local: int, nx: int, ny: int, variants=PE
         out[f"d2q{lattice}_{storage}"] = {
             "lattice": f"D2Q{lattice}", "storage": storage, "dtype": DTYPE[storage],
             "steps": steps, "ms_per_step": t / steps * 1e3, "mlups": N * steps / t / 1e6,
-            "roofline": roofline_of(torch, local, lattice, storage, N, steps, t, clocks),
+            "roofline": roofline_of(torch, local, lattice, storage, N, steps, t, clocks, lay),
             "launch": {k: lay[k] for k in ("tile_rows", "grid_x", "grid_y", "stages")},
             "clocks": clocks}
     return out
@@ -492,7 +500,7 @@ def run_gpu(args, world, rank, local):
     # ---- roofline of the fused kernel ----------------------------------------
     clocks = clk.summary()
     roofline = roofline_of(torch, local, args.lattice, args.storage, N, args.steps, t_local,
-                           clocks)
+                           clocks, lay)
     sim.close()
     if rank != 0:
         return 0
@@ -513,7 +521,7 @@ def run_gpu(args, world, rank, local):
                 "h2d_bytes_per_step": 3 * N * 8, "d2h_bytes_per_step": 3 * N * 8,
                 "lbm_steps_per_e2e_step": lbm_per_e2e, "e2e_steps": n_e2e,
                 "path": "Simulation.set_equilibrium(pinned rho,u) -> step -> moments(pinned)"},
-        "gpu_launches": args.steps,
+        "gpu_launches": -(-args.steps // steps_per_launch(lay, args.lattice, args.storage)),
         "clocks": clocks,
     }
     if not args.no_per_storage:

@@ -151,7 +151,8 @@ int lbm_set_populations(lbm_ctx* c, const double* f);
 int lbm_set_equilibrium(lbm_ctx* c, const double* rho, const double* ux, const double* uy,
                         const double* dfi);
 
-/* Advances nsteps >= 0 time steps (one fused kernel launch per step): the
+/* Advances nsteps >= 0 time steps (one fused kernel launch per step, or per two
+ * steps where both fit one launch; the values are the same): the
  * update of Sec. II per node -- streaming, Eqs. M0 and M1, psi (Eq. EOS or
  * the exponential form), F_FF (Eq. force_SC), F_FS and Delta F_S (Eqs.
  * force_SC_FS, wall_shift), the optional projection (after Eq. f2) and the
@@ -223,8 +224,9 @@ const char* lbm_last_error(const lbm_ctx* c);
 int lbm_debug_stall_next_step(lbm_ctx* c, int32_t wait_ms);
 
 /* Layout facts for measurement: bytes per node per step that the population
- * traffic needs (2 Q s), the padded row pitch in elements, and the launch shape
- * (strip width, rows per CTA, grid) of the fused step. */
+ * traffic needs (2 Q s, halved where a launch advances two steps), the padded
+ * row pitch in elements, and the launch shape of consecutive steps (columns and
+ * rows per CTA, grid, load stages). */
 typedef struct {
   int64_t bytes_per_node;
   int64_t pitch;

@@ -30,7 +30,13 @@ struct lbm_ctx {
   int64_t pitch = 0, rows = 0, plane = 0;
   void* buf[2] = {nullptr, nullptr};
   int cur = 0;  // buffer holding the current state
-  PopMaps tmap[2];       // population maps of buffer 0 and 1 (one per box depth)
+  PopMaps tmap[2];       // population maps of buffer 0 and 1 (one per box depth): row march
+  // Tile shapes (launch.cuh: tile_list) of one step (-1: the row march), of two
+  // steps per launch (-1: none) and of the read-out, with their maps per buffer.
+  enum { kOne, kTwo, kRead, kTiles };
+  int shape[kTiles] = {-1, -1, -1};
+  PopMaps tile_map[kTiles][2];  // encoded on first use
+  bool tile_ready[kTiles] = {false, false, false};
   // wall (compute precision: double for FP64 storage, float otherwise)
   void* wall_phie = nullptr;
   void* wall_sx = nullptr;
@@ -195,6 +201,68 @@ template <int Q, typename S> int make_tmap(lbm_ctx* c, int which) {
   return LBM_OK;
 }
 
+// Maps of tile use `use` (kOne, kTwo, kRead) for both population buffers.
+template <int Q, typename S> int ready_tile_maps(lbm_ctx* c, int use) {
+  if (c->shape[use] < 0 || c->tile_ready[use]) return LBM_OK;
+  EncodeFn enc = get_encode();
+  if (!enc) return fail(c, LBM_ECUDA, "cuTensorMapEncodeTiled entry point unavailable");
+  const TileInfo t = tile_info<Q, S>(c->shape[use]);
+  if (t.slots <= 0) return fail(c, LBM_ECUDA, "tile kernel cannot be resident (%s)", cudaGetErrorString(cudaGetLastError()));
+  cuuint64_t dims[3] = {(cuuint64_t)(c->p.nx + 2 * c->GX), (cuuint64_t)c->rows, (cuuint64_t)Q};
+  cuuint64_t strides[2] = {(cuuint64_t)(c->pitch * sizeof(S)), (cuuint64_t)(c->plane * sizeof(S))};
+  cuuint32_t estr[3] = {1, 1, 1};
+  for (int b = 0; b < 2; ++b) {
+    c->tile_map[use][b] = PopMaps{};
+    for (int k = 0; k < t.nmap; ++k) {
+      cuuint32_t box[3] = {(cuuint32_t)t.bw, (cuuint32_t)t.bh, (cuuint32_t)t.depth[k]};
+      CUresult r = enc(&c->tile_map[use][b].m[k], tma_type<S>(), 3, c->buf[b], dims, strides, box,
+                       estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS) return fail(c, LBM_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+    }
+  }
+  c->tile_ready[use] = true;
+  return LBM_OK;
+}
+
+// Estimated microseconds per launch of tile shape k on the given lattices: the
+// rounds of resident CTAs it takes, the last one counted whole while there are
+// few, plus the launch and the first loads.
+template <int Q, typename S> double tile_cost(int k, int64_t tiles) {
+  const TileInfo t = tile_info<Q, S>(k);
+  if (t.slots <= 0) return 1e30;
+  const double r = (double)tiles / t.slots;
+  return 1.2 + tile_list<Q, S>().t[k].us * (r < 4.0 ? std::ceil(r) : r + 0.5);
+}
+
+// Picks the tile shapes of a lattice, all by estimated time per step.  One row
+// march stays ahead of the one-step tiles: D2Q9 FP32 on lattices whose two
+// buffers exceed L2 twice over, which HBM bounds (8192x4096: 0.368 ms against
+// 0.399; 4096x2048: 0.0963 against 0.0983).  Two steps per launch need whole node pairs under
+// periodic wrapping (even nx) and a lattice no smaller than the halo; an
+// explicit tile_rows asks for the row march.
+template <int Q, typename S> void choose_tiles(lbm_ctx* c) {
+  constexpr TileList list = tile_list<Q, S>();
+  c->shape[lbm_ctx::kRead] = list.moments;
+  if (c->p.tile_rows > 0) return;
+  const int64_t nodes = (int64_t)c->p.nx * c->p.ny;
+  const bool march = Q == 9 && sizeof(S) == 4 && 2 * Q * (int64_t)sizeof(S) * nodes > (int64_t)260 << 20;
+  double best[2] = {1e30, 1e30};
+  for (int k = 0; k < list.n; ++k) {
+    const TileCfg& t = list.t[k];
+    const int use = t.steps == 2 ? lbm_ctx::kTwo : lbm_ctx::kOne;
+    if (use == lbm_ctx::kTwo && (c->p.nx % 2 || c->p.nx < 4 || c->p.ny < 4)) continue;
+    if (use == lbm_ctx::kOne && march) continue;
+    const int64_t tiles = (int64_t)((c->p.nx + t.tw - 1) / t.tw) * ((c->p.ny + t.th - 1) / t.th);
+    const double us = tile_cost<Q, S>(k, tiles) / t.steps;
+    if (us < best[use]) {
+      best[use] = us;
+      c->shape[use] = k;
+    }
+  }
+  if (!march && best[lbm_ctx::kTwo] >= best[lbm_ctx::kOne]) c->shape[lbm_ctx::kTwo] = -1;
+}
+
 // Rows per CTA segment.  Measured on GB300 (8192x4096 D2Q9 sweep): short
 // segments run fastest -- many waves of short CTAs keep the concurrently
 // active tiles in a compact band of rows and balance the SMs dynamically; with
@@ -234,6 +302,7 @@ template <int Q, typename S> int setup_layout(lbm_ctx* c) {
     int rc = make_tmap<Q, S>(c, b);
     if (rc) return rc;
   }
+  choose_tiles<Q, S>(c);
   int dev = 0, sms = 0;
   CK(c, cudaGetDevice(&dev));
   CK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -310,13 +379,28 @@ StepArgs<typename Codec<S>::T, S> make_args(const lbm_ctx* c, int src, S* fout, 
   return a;
 }
 
+// Enqueues the read-out pass over the current buffer.
 template <int Q, typename S>
-int run_pass(lbm_ctx* c, int mode, double* o_rho, double* o_ux, double* o_uy, int momentum,
-             S* fout) {
-  const auto a = make_args<Q, S>(c, c->cur, fout, o_rho, o_ux, o_uy, momentum);
+int run_moments(lbm_ctx* c, double* o_rho, double* o_ux, double* o_uy, int momentum) {
+  if (int rc = ready_tile_maps<Q, S>(c, lbm_ctx::kRead)) return rc;
+  const auto a = make_args<Q, S>(c, c->cur, nullptr, o_rho, o_ux, o_uy, momentum);
+  CK(c, launch_tile<Q, S>(c->shape[lbm_ctx::kRead], c->tile_map[lbm_ctx::kRead][c->cur], c->wall_flags,
+                          c->nchunk_pad, a, c->stream, kModeMoments));
+  return LBM_OK;
+}
+
+// Enqueues one launch of `use` (kOne or kTwo steps) into the other buffer.
+template <int Q, typename S> int run_steps(lbm_ctx* c, int use) {
+  if (int rc = ready_tile_maps<Q, S>(c, use)) return rc;
+  const auto a = make_args<Q, S>(c, c->cur, static_cast<S*>(c->buf[c->cur ^ 1]), nullptr, nullptr, nullptr, 0);
+  if (c->shape[use] >= 0) {
+    CK(c, launch_tile<Q, S>(c->shape[use], c->tile_map[use][c->cur], c->wall_flags, c->nchunk_pad, a,
+                            c->stream, kModeStep));
+    return LBM_OK;
+  }
   // Without walls the flag map is never read; the population map stands in.
   const CUtensorMap& fm = c->has_wall ? c->flag_map : c->tmap[c->cur].m[0];
-  CK(c, launch_step<Q, S>(c->tmap[c->cur], fm, a, dim3(c->grid_x, c->grid_y), c->stream, mode));
+  CK(c, launch_step<Q, S>(c->tmap[c->cur], fm, a, dim3(c->grid_x, c->grid_y), c->stream));
   return LBM_OK;
 }
 
@@ -585,15 +669,19 @@ int lbm_step(lbm_ctx* c, int64_t nsteps) {
   if (rc) return rc;
   if (nsteps < 0) return fail(c, LBM_EINVAL, "negative step count");
   if (!c->has_state) return fail(c, LBM_ESTATE, "populations not set");
-  for (int64_t s = 0; s < nsteps; ++s) {
+  for (int64_t s = 0; s < nsteps;) {
+    // Two steps in one launch unless a check falls between them (or the test
+    // hook, which covers one step, is armed).
+    const bool two = c->shape[lbm_ctx::kTwo] >= 0 && s + 2 <= nsteps && !c->stall_wait_ns &&
+                     (c->p.check_every <= 0 || (c->steps + 1) % c->p.check_every != 0);
     rc = dispatch(c->Q, c->p.storage, [&]<int Q, typename S>() -> int {
-      return run_pass<Q, S>(c, kModeStep, nullptr, nullptr, nullptr, 0,
-                            static_cast<S*>(c->buf[c->cur ^ 1]));
+      return run_steps<Q, S>(c, two ? lbm_ctx::kTwo : lbm_ctx::kOne);
     });
     if (rc) return rc;
-    c->stall_wait_ns = 0;  // the test hook covers one step
+    c->stall_wait_ns = 0;
     c->cur ^= 1;
-    c->steps += 1;
+    s += two ? 2 : 1;
+    c->steps += two ? 2 : 1;
     if (c->p.check_every > 0 && c->steps % c->p.check_every == 0) {
       rc = read_status(c);
       if (rc) return rc;
@@ -612,8 +700,7 @@ int lbm_moments_device(lbm_ctx* c, double* d_rho, double* d_ux, double* d_uy) {
   double* sink = scratch.as<double>();
   if ((!d_rho || !d_ux || !d_uy) && !sink) return fail(c, LBM_ENOMEM, "moments scratch");
   return dispatch(c->Q, c->p.storage, [&]<int Q, typename S>() -> int {
-    return run_pass<Q, S>(c, kModeMoments, d_rho ? d_rho : sink, d_ux ? d_ux : sink,
-                          d_uy ? d_uy : sink, 0, nullptr);
+    return run_moments<Q, S>(c, d_rho ? d_rho : sink, d_ux ? d_ux : sink, d_uy ? d_uy : sink, 0);
   });
 }
 
@@ -665,7 +752,7 @@ int lbm_totals(lbm_ctx* c, double out[3]) {
   if (!stage.p) return fail(c, LBM_ENOMEM, "totals staging");
   double* d = stage.as<double>();
   rc = dispatch(c->Q, c->p.storage, [&]<int Q, typename S>() -> int {
-    return run_pass<Q, S>(c, kModeMoments, d, d + N, d + 2 * N, 1, nullptr);
+    return run_moments<Q, S>(c, d, d + N, d + 2 * N, 1);
   });
   if (rc) return rc;
   CK(c, launch_reduce3(d, d + N, d + 2 * N, N, c->d_partials, c->nparts, c->d_out3, c->stream));
@@ -738,13 +825,30 @@ int lbm_debug_stall_next_step(lbm_ctx* c, int32_t wait_ms) {
 
 int lbm_get_layout(const lbm_ctx* c, lbm_layout* out) {
   if (!c || !out) return fail(nullptr, LBM_EINVAL, "null argument");
-  out->bytes_per_node = 2LL * c->Q * c->esize;
+  const int use = c->shape[lbm_ctx::kTwo] >= 0 ? lbm_ctx::kTwo : lbm_ctx::kOne;
+  out->bytes_per_node = 2LL * c->Q * c->esize / (use == lbm_ctx::kTwo ? 2 : 1);
   out->pitch = c->pitch;
-  out->strip_width = c->W;
-  out->tile_rows = c->tile_rows;
-  out->grid_x = c->grid_x;
-  out->grid_y = c->grid_y;
-  out->stages = c->NS;
+  if (c->shape[use] >= 0) {
+    const TileCfg t = [&] {
+      TileCfg v{};
+      dispatch(c->Q, c->p.storage, [&]<int Q, typename S>() -> int {
+        v = tile_list<Q, S>().t[c->shape[use]];
+        return LBM_OK;
+      });
+      return v;
+    }();
+    out->strip_width = t.tw;
+    out->tile_rows = t.th;
+    out->grid_x = (c->p.nx + t.tw - 1) / t.tw;
+    out->grid_y = (c->p.ny + t.th - 1) / t.th;
+    out->stages = 1;
+  } else {
+    out->strip_width = c->W;
+    out->tile_rows = c->tile_rows;
+    out->grid_x = c->grid_x;
+    out->grid_y = c->grid_y;
+    out->stages = c->NS;
+  }
   out->ghost_x = c->GX;
   out->ghost_y = c->GY;
   out->device_bytes = 2LL * c->plane * c->Q * c->esize;

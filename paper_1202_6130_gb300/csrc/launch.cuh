@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "step_kernel.cuh"
+#include "tile_kernel.cuh"
 
 namespace lbm {
 
@@ -45,11 +46,61 @@ template <int Q, typename S> struct StepConfig {
 template <int Q, typename S>
 using ConfigShape = StepShape<Q, S, StepConfig<Q, S>::W, StepConfig<Q, S>::NS>;
 
-// Launches the fused step (mode kModeStep) or the read-out pass (kModeMoments).
+// Launches the fused step as a row march.
 template <int Q, typename S>
 cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
                         const StepArgs<typename Codec<S>::T, S>& a, dim3 grid,
-                        cudaStream_t stream, int mode);
+                        cudaStream_t stream);
+
+// Shapes of the tile kernel per (lattice, storage): tile width and height,
+// threads, time steps per launch, whether tiles without edges or walls run a
+// copy of the update without that code, CTAs per SM the registers are sized
+// for, and the microseconds one round of resident CTAs takes (GB300, lattices
+// of 2048x1024 and larger).  choose_tiles picks the shape with the least
+// estimated time, rounds x this figure, per time step.
+struct TileCfg {
+  int tw, th, nt, steps;
+  bool in;
+  int minb;
+  double us;
+};
+constexpr int kMaxTileShapes = 6;
+struct TileList {
+  TileCfg t[kMaxTileShapes];
+  int n;
+  int moments;  // the shape that also reads out the moments
+};
+template <int Q, typename S> constexpr TileList tile_list() {
+  if constexpr (sizeof(S) == 8 && Q == 9)
+    return {{{16, 4, 64, 1, false, 4, 18.0}, {32, 8, 256, 1, false, 3, 29.7}, {32, 16, 256, 1, true, 2, 38.4}}, 3, 2};
+  else if constexpr (sizeof(S) == 8)
+    return {{{16, 4, 64, 1, false, 4, 48.0}, {32, 8, 256, 1, false, 3, 62.0}, {32, 16, 256, 1, true, 2, 80.0}}, 3, 2};
+  else if constexpr (Q == 21 && sizeof(S) == 4)
+    return {{{16, 4, 64, 1, false, 4, 3.0}, {32, 8, 256, 1, false, 3, 4.3}, {64, 8, 256, 1, true, 2, 5.2}}, 3, 1};
+  else if constexpr (Q == 21)
+    return {{{32, 4, 64, 1, false, 8, 4.1}, {64, 8, 128, 1, true, 4, 6.9}}, 2, 1};
+  else if constexpr (sizeof(S) == 4)
+    return {{{32, 4, 64, 1, false, 8, 2.8}, {64, 8, 128, 1, true, 7, 6.4}}, 2, 0};
+  else
+    return {{{32, 4, 64, 1, false, 8, 2.5}, {64, 8, 128, 1, true, 7, 4.1}}, 2, 0};
+}
+template <int Q, typename S, int K> struct TileConfig {
+  static constexpr TileCfg kCfg = tile_list<Q, S>().t[K];
+  using Sh = TileShape<Q, S, kCfg.tw, kCfg.th, kCfg.nt, kCfg.steps, kCfg.in>;
+};
+
+// Launches tile shape `shape`: its steps (kModeStep), or the read-out pass
+// (kModeMoments; the list's `moments` shape only).
+template <int Q, typename S>
+cudaError_t launch_tile(int shape, const PopMaps& src, const uint32_t* flags, int flag_pitch,
+                        const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream, int mode);
+
+// What the host needs of a tile shape: its TMA boxes, and the tiles that one
+// round of resident CTAs takes (0 if the kernel cannot run).
+struct TileInfo {
+  int bw, bh, nmap, depth[kMaxMaps], slots;
+};
+template <int Q, typename S> TileInfo tile_info(int shape);
 
 // CTAs of the step kernel that fit on one SM (occupancy query).
 template <int Q, typename S> int step_ctas_per_sm();

@@ -365,6 +365,9 @@ __device__ __forceinline__ void node_moments(const T (&f)[Q], T& rho, T& jx, T& 
   }
 }
 
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return a * b; }
+
 // Total force on a node (Eqs. force_SC, force_SC_FS, wall_shift):
 //   F = F_FF + rho S + rho phi^eps (U_wall - u - F_FF / rho) + body force.
 // sfx, sfy: sum_i w_i psi(x + r_i) r_i; wall terms only when has_wall.
@@ -373,8 +376,10 @@ __device__ __forceinline__ void node_force(const Physics<T>& P, T rho, T ux, T u
                                            T sfx, T sfy, bool has_wall, T phie, T Sx, T Sy,
                                            T uwx, T uwy, T inv_rho, T& Fx, T& Fy) {
   const T mg = -P.G * psi_c;
-  const T ffx = mg * sfx;
-  const T ffy = mg * sfy;
+  // Rounded products in FP32: the same bits whether or not a kernel holds the
+  // wall terms (which decide what the compiler could fuse).
+  const T ffx = mul_rn(mg, sfx);
+  const T ffy = mul_rn(mg, sfy);
   Fx = ffx;
   Fy = ffy;
   if (has_wall) {

@@ -6,12 +6,18 @@
 
 namespace lbm {
 
-template <int Q, typename S, int MODE, int FL>
+// The common settings (exponential psi, no projection, stochastic rounding of
+// 16-bit storage) run kernels with them fixed at compile time.
+template <typename T, typename S> static bool plain_flags(const StepArgs<T, S>& a) {
+  return a.phys.psi_kind == 0 && !a.phys.project && (a.stochastic || !Codec<S>::kShifted);
+}
+
+template <int Q, typename S, int FL>
 static cudaError_t prepare_kernel() {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
   static cudaError_t once = cudaFuncSetAttribute(
-      step_kernel<Q, S, Cfg::W, Cfg::NS, MODE, Cfg::MINB, FL>,
+      step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, FL>,
       cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
   return once;
 }
@@ -26,7 +32,7 @@ static cudaError_t launch_step_pdl(const PopMaps& src, const CUtensorMap& flags,
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
   cudaError_t e;
-  if ((e = prepare_kernel<Q, S, kModeStep, FL>()) != cudaSuccess) return e;
+  if ((e = prepare_kernel<Q, S, FL>()) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(Sh::NT);
@@ -37,40 +43,94 @@ static cudaError_t launch_step_pdl(const PopMaps& src, const CUtensorMap& flags,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, step_kernel<Q, S, Cfg::W, Cfg::NS, kModeStep, Cfg::MINB, FL>,
+  return cudaLaunchKernelEx(&cfg, step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, FL>,
                             src, flags, a);
 }
 
 template <int Q, typename S>
 cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
                         const StepArgs<typename Codec<S>::T, S>& a, dim3 grid,
-                        cudaStream_t stream, int mode) {
-  using Cfg = StepConfig<Q, S>;
-  using Sh = ConfigShape<Q, S>;
-  cudaError_t e;
-  if (mode == kModeStep) {
-    // The common settings (exponential psi, no projection, stochastic
-    // rounding of 16-bit storage) run a kernel with them fixed at compile time.
-    const bool plain = a.phys.psi_kind == 0 && !a.phys.project &&
-                       (a.stochastic || !Codec<S>::kShifted);
-    e = plain ? launch_step_pdl<Q, S, kFlExpPlain>(src, flags, a, grid, stream)
-              : launch_step_pdl<Q, S, kFlRuntime>(src, flags, a, grid, stream);
-    if (e != cudaSuccess) return e;
-  } else {
-    if ((e = prepare_kernel<Q, S, kModeMoments, kFlRuntime>()) != cudaSuccess) return e;
-    step_kernel<Q, S, Cfg::W, Cfg::NS, kModeMoments, Cfg::MINB, kFlRuntime>
-        <<<grid, Sh::NT, Sh::SMEM, stream>>>(src, flags, a);
-  }
-  return cudaGetLastError();
+                        cudaStream_t stream) {
+  return plain_flags(a) ? launch_step_pdl<Q, S, kFlExpPlain>(src, flags, a, grid, stream)
+                        : launch_step_pdl<Q, S, kFlRuntime>(src, flags, a, grid, stream);
+}
+
+template <int Q, typename S, int K, int MODE, int FL>
+static cudaError_t prepare_tile() {
+  using Cfg = TileConfig<Q, S, K>;
+  static cudaError_t once = cudaFuncSetAttribute(tile_kernel<typename Cfg::Sh, MODE, FL, Cfg::kCfg.minb>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 Cfg::Sh::SMEM);
+  return once;
+}
+
+template <int Q, typename S, int K, int MODE, int FL>
+static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int flag_pitch,
+                                 const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream) {
+  using Cfg = TileConfig<Q, S, K>;
+  using Sh = typename Cfg::Sh;
+  cudaError_t e = prepare_tile<Q, S, K, MODE, FL>();
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW, (a.ny + Sh::TH - 1) / Sh::TH);
+  cfg.blockDim = dim3(Sh::NT);
+  cfg.dynamicSmemBytes = Sh::SMEM;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, tile_kernel<Sh, MODE, FL, Cfg::kCfg.minb>, src, flags, flag_pitch, a);
+}
+
+// Calls fn<K>() for the K-th shape of the list.
+template <int Q, typename S, int K = 0, typename F> auto with_shape(int shape, F&& fn) {
+  if constexpr (K + 1 < tile_list<Q, S>().n)
+    if (shape != K) return with_shape<Q, S, K + 1>(shape, fn);
+  return fn.template operator()<K>();
+}
+
+template <int Q, typename S>
+cudaError_t launch_tile(int shape, const PopMaps& src, const uint32_t* flags, int flag_pitch,
+                        const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream, int mode) {
+  if (mode == kModeMoments)
+    return launch_tile_k<Q, S, tile_list<Q, S>().moments, kModeMoments, kFlRuntime>(
+        src, flags, flag_pitch, a, stream);
+  return with_shape<Q, S>(shape, [&]<int K>() {
+    return plain_flags(a) ? launch_tile_k<Q, S, K, kModeStep, kFlExpPlain>(src, flags, flag_pitch, a, stream)
+                          : launch_tile_k<Q, S, K, kModeStep, kFlRuntime>(src, flags, flag_pitch, a, stream);
+  });
+}
+
+template <int Q, typename S> TileInfo tile_info(int shape) {
+  return with_shape<Q, S>(shape, [&]<int K>() {
+    using Cfg = TileConfig<Q, S, K>;
+    using Sh = typename Cfg::Sh;
+    TileInfo t{Sh::BW, Sh::BH, Sh::NMAP, {}, 0};
+    for (int k = 0; k < Sh::NMAP; ++k) t.depth[k] = Sh::kTab.depth[k];
+    static int slots = [] {
+      int n = 0, dev = 0, sms = 0;
+      if (prepare_tile<Q, S, K, kModeStep, kFlExpPlain>() != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+              &n, tile_kernel<Sh, kModeStep, kFlExpPlain, Cfg::kCfg.minb>, Sh::NT, Sh::SMEM) != cudaSuccess ||
+          cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+      return n * sms;
+    }();
+    t.slots = slots;
+    return t;
+  });
 }
 
 template <int Q, typename S> int step_ctas_per_sm() {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
-  if (prepare_kernel<Q, S, kModeStep, kFlRuntime>() != cudaSuccess) return 0;
+  if (prepare_kernel<Q, S, kFlRuntime>() != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &n, step_kernel<Q, S, Cfg::W, Cfg::NS, kModeStep, Cfg::MINB, kFlRuntime>, Sh::NT,
+          &n, step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, kFlRuntime>, Sh::NT,
           Sh::SMEM) != cudaSuccess)
     return 0;
   return n;
@@ -145,7 +205,9 @@ template <int Q, typename S> int batch_ctas_per_sm() {
 #define LBM_INSTANTIATE_STEP(Q, S)                                                         \
   template cudaError_t lbm::launch_step<Q, S>(const PopMaps&, const CUtensorMap&,      \
                                               const lbm::StepArgs<lbm::Codec<S>::T, S>&,   \
-                                              dim3, cudaStream_t, int);                    \
+                                              dim3, cudaStream_t);                         \
+  template cudaError_t lbm::launch_tile<Q, S>(int, const PopMaps&, const uint32_t*, int, const lbm::StepArgs<lbm::Codec<S>::T, S>&, cudaStream_t, int); \
+  template lbm::TileInfo lbm::tile_info<Q, S>(int); \
   template int lbm::step_ctas_per_sm<Q, S>();                                            \
   template cudaError_t lbm::launch_batch<Q, S>(                                          \
       const lbm::BatchArgs<lbm::Codec<S>::T, S>&,                                         \

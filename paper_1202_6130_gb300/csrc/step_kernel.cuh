@@ -34,67 +34,11 @@
 #include "f2.cuh"
 #include "lattice.cuh"
 #include "node.cuh"
+#include "node_update.cuh"
+#include "step_args.cuh"
 #include "tma.cuh"
 
 namespace lbm {
-
-enum : uint32_t { kStatusNonFinite = 1u, kStatusTimeout = 2u };
-
-enum StepMode : int {
-  kModeStep = 0,      // write post-collision populations to fout
-  kModeMoments = 1,   // write rho and u = (j + F/2) / rho (FP64) instead
-};
-
-// Which run-time switches of the update are fixed at compile time:
-// kFlRuntime reads psi_kind, project and the rounding mode from the
-// arguments; kFlExpPlain is the exponential pseudo-potential without the
-// projection step, with stochastic rounding for 16-bit storage (the other
-// settings run the kFlRuntime kernel).  Both give the same bits.
-enum StepFlags : int { kFlRuntime = 0, kFlExpPlain = 1 };
-
-template <typename T, typename S> struct StepArgs {
-  Physics<T> phys;
-  WallFields<T> wall;
-  int32_t nx, ny;
-  int32_t pitch;       // elements per padded row
-  int32_t tile_rows;   // L
-  int64_t plane;       // elements per population plane
-  S* fout;             // kModeStep: destination buffer (same layout as the source)
-  double* out_rho;     // kModeMoments: [ny][nx]
-  double* out_ux;
-  double* out_uy;
-  int32_t momentum;    // kModeMoments: 1 -> out_ux/out_uy get j + F/2 instead of u
-  uint32_t* status;    // error bits (kStatus*)
-  uint64_t wait_ns;    // bound of every stage wait
-  uint32_t extra_tx;   // test hook: bytes each stage expects beyond its copies (0 normally)
-  // Step counter of the stochastic rounding: two words indexed by the source
-  // buffer; a step reads rng[rng_idx] and one CTA writes rng[rng_idx ^ 1] =
-  // rng[rng_idx] + 1 for the next step (kModeStep only).
-  uint32_t* rng;
-  int32_t rng_idx;
-  int32_t stochastic;  // 16-bit storage: 1 = stochastic rounding, 0 = nearest-even
-};
-
-// Counter of the step about to run (0 unless it is needed).
-template <typename S, int MODE, int FL, typename Args>
-__device__ __forceinline__ uint32_t step_key(const Args& a) {
-  if constexpr (MODE == kModeStep && Codec<S>::kShifted) {
-    if (FL == kFlExpPlain || a.stochastic) return a.rng[a.rng_idx];
-  }
-  return 0u;
-}
-
-// Advances the counter for the next step; called by one thread of one CTA.
-template <int MODE, typename Args> __device__ __forceinline__ void advance_key(const Args& a) {
-  if constexpr (MODE == kModeStep) a.rng[a.rng_idx ^ 1] = a.rng[a.rng_idx] + 1u;
-}
-
-// TMA maps of one population buffer, one per distinct box depth of the
-// lattice's plane groups (D2Q9 uses one, D2Q21 three).
-constexpr int kMaxMaps = 3;
-struct PopMaps {
-  CUtensorMap m[kMaxMaps];
-};
 
 template <int Q, typename S, int W, int NS> struct StepShape {
   using L = Lattice<Q>;
@@ -241,7 +185,7 @@ __device__ __forceinline__ uint64_t step_smem_init(const StepSmem<Q, S, W, NS>& 
 // `rev` the segment is marched upwards (row y0 + Lr + R - 1 first); the node
 // arithmetic is the same in either direction.  Returns false if a stage never
 // arrived (the status word then has kStatusTimeout).
-template <int Q, typename S, int W, int NS, int MODE, int FL, typename Args>
+template <int Q, typename S, int W, int NS, int FL, typename Args>
 __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensorMap* flg,
                                               const Args& a, int x0, int y0, int Lr, bool rev,
                                               const StepSmem<Q, S, W, NS>& sm, uint32_t& g,
@@ -394,114 +338,11 @@ __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensor
         });
         flag = flags_of(sto);
       }
-      T rho, jx, jy;
-      node_moments<Q, T>(f, rho, jx, jy);
-      const T inv_rho = rcp_node<S, T>(rho);
-      const T ux = div_rho<T>(jx, rho, inv_rho);
-      const T uy = div_rho<T>(jy, rho, inv_rho);
-
-      // sum_i w_i psi(x + c_i) c_i from the ring (rest state contributes 0).
-      // prow[R + c_y]: the ring row of node row yo + c_y, at this thread's column.
-      static_assert((Sh::RING_H & (Sh::RING_H - 1)) == 0, "ring height is a power of two");
-      const T* prow[2 * R + 1];
-      static_for<0, 2 * R + 1>([&](auto rc) {
-        constexpr int cy = decltype(rc)::value - R;
-        prow[R + cy] = ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + tid + Sh::RO;
-      });
-      const T psi_c = prow[R][0];
-      T sfx = 0, sfy = 0;
-      static_for<0, Q>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        if constexpr (L::cx(i) != 0 || L::cy(i) != 0) {
-          const T nb = prow[R + L::cy(i)][L::cx(i)];
-          const T wn = T(L::w(i)) * nb;
-          if constexpr (L::cx(i) != 0) sfx += cmul<L::cx(i)>(wn);
-          if constexpr (L::cy(i) != 0) sfy += cmul<L::cy(i)>(wn);
-        }
-      });
-
-      // Wall terms only on flagged (row, 32-column chunk) pairs.
-      const bool has_wall = flag != 0u && x < a.nx;
-      T phie = 0, Sx = 0, Sy = 0, uwx = 0, uwy = 0;
-      if (has_wall) {
-        const int64_t n = (int64_t)yo * a.nx + x;
-        phie = a.wall.phie[n];
-        Sx = a.wall.sx[n];
-        Sy = a.wall.sy[n];
-        if (a.wall.uwx) {
-          uwx = a.wall.uwx[n];
-          uwy = a.wall.uwy[n];
-        }
-      }
-      T Fx, Fy;
-      node_force<T>(a.phys, rho, ux, uy, psi_c, sfx, sfy, has_wall, phie, Sx, Sy, uwx, uwy,
-                    inv_rho, Fx, Fy);
-
-      if (x < a.nx) {
-        if (!(fabs(rho) <= T(3.0e38))) atomicOr(a.status, kStatusNonFinite);
-        if constexpr (MODE == kModeStep) {
-          const T usx = ux + div_rho<T>(Fx, rho, inv_rho);
-          const T usy = uy + div_rho<T>(Fy, rho, inv_rho);
-          if (FL != kFlExpPlain && a.phys.project) project<Q, T>(f, rho, jx, jy);
-          node_collide<Q, T>(a.phys, f, rho, ux, uy, usx, usy);
-          // The primary store plus periodic images inside the ghost frame.
-          S e[Q];
-#pragma unroll
-          for (int i = 0; i < Q; ++i) e[i] = C::store_rn(f[i]);
-          S* out = a.fout + (int64_t)(yo + GY) * a.pitch + x + GX;
-          static_for<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            out[Planes<Q>::template plane<i> * a.plane] = e[i];
+      node_update<Q, S, kModeStep, FL>(
+          a, f, flag, x, yo, strip_edge, simple_images,
+          [&](int cy) -> const T* {  // ring row of node row yo + c_y
+            return ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + tid + Sh::RO;
           });
-          // Periodic images exist only for nodes within GX of a side or GY of
-          // the top or bottom; the strip test is per CTA, the row test per row.
-          const bool xedge = strip_edge && (x < GX || x >= a.nx - GX);
-          const bool yedge = yo < GY || yo >= a.ny - GY;
-          if ((xedge || yedge) && simple_images) {
-            // at most one image column (+-nx) and one image row (+-ny)
-            const int sx = !xedge ? 0 : (x < GX ? a.nx : -a.nx);
-            const int64_t sy = !yedge ? 0 : (int64_t)(yo < GY ? a.ny : -a.ny) * a.pitch;
-            auto put = [&](int64_t d) {
-              static_for<0, Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                out[d + Planes<Q>::template plane<i> * a.plane] = e[i];
-              });
-            };
-            if (sx != 0) put(sx);
-            if (sy != 0) {
-              put(sy);
-              if (sx != 0) put(sy + sx);
-            }
-          } else if (xedge || yedge) {
-            int xa = x;
-            while (xa - a.nx >= -GX) xa -= a.nx;
-            int ya = yo;
-            while (ya - a.ny >= -GY) ya -= a.ny;
-            for (int ym = ya; ym < a.ny + GY; ym += a.ny) {
-              for (int xm = xa; xm < a.nx + GX; xm += a.nx) {
-                if (xm == x && ym == yo) continue;
-                S* o2 = a.fout + (int64_t)(ym + GY) * a.pitch + xm + GX;
-                static_for<0, Q>([&](auto ic) {
-                  constexpr int i = decltype(ic)::value;
-                  o2[Planes<Q>::template plane<i> * a.plane] = e[i];
-                });
-              }
-            }
-          }
-        } else {
-          const int64_t n = (int64_t)yo * a.nx + x;
-          const double px = (double)jx + 0.5 * (double)Fx;
-          const double py = (double)jy + 0.5 * (double)Fy;
-          a.out_rho[n] = (double)rho;
-          if (a.momentum) {
-            a.out_ux[n] = px;
-            a.out_uy[n] = py;
-          } else {
-            a.out_ux[n] = px / (double)rho;
-            a.out_uy[n] = py / (double)rho;
-          }
-        }
-      }
     }
     if (++s == NS) {
       s = 0;
@@ -537,13 +378,12 @@ __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensor
 // (D2Q21) the collision re-reads them from the row's stage, as march_segment
 // does.  Wall terms, ghost images, the halo psi and a pair that straddles the
 // lattice's right edge fall back to per-node code.
-template <int Q, typename S, int W, int NS, int MODE, int FL, typename Args>
+template <int Q, typename S, int W, int NS, int FL, typename Args>
 __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUtensorMap* flg,
                                                  const Args& a, int x0, int y0, int Lr, bool rev,
                                                  const StepSmem<Q, S, W, NS>& sm, uint32_t& g) {
   using Sh = StepShape<Q, S, W, NS>;
   using L = Lattice<Q>;
-  using E = EqConst<Q>;
   using C = Codec<S>;
   using PR = Pair<S>;
   using T = float;
@@ -576,7 +416,7 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
   const bool simple_images = a.nx >= 2 * GX && a.ny >= 2 * GY && (a.nx & 1) == 0;
   const uint32_t tx_bytes = Sh::TX_POP + (wall_on ? Sh::TX_FLAGS : 0u) + a.extra_tx;
   constexpr int kIss = kIssuer<Sh::NT>;
-  const uint32_t key = step_key<S, MODE, FL>(a);
+  const uint32_t key = step_key<S, kModeStep, FL>(a);
 
   __syncthreads();
 
@@ -619,17 +459,6 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
       return PR::load1(st[off + xc], st[off + xc + 1]);
     }
   };
-  // rho from the sum H of a node's stored values: H itself, or for 16-bit
-  // storage H / sigma + rho_s (the shifts w_i rho_s sum to rho_s).
-  constexpr T kInvScale = T(1) / T(C::kScale);
-  auto rho_of = [&](T H) -> T {
-    if constexpr (C::kShifted) return fmaf(H, kInvScale, a.phys.rho_s);
-    else return H;
-  };
-  auto rho_of2 = [&](F2 H) -> F2 {
-    if constexpr (C::kShifted) return fma2(H, F2::splat(kInvScale), F2::splat(a.phys.rho_s));
-    else return H;
-  };
   auto psi_at = [&](const S* st, int xl) -> T {  // one node (halo columns)
     T H = 0;
     static_for<0, Q>([&](auto ic) {
@@ -638,7 +467,7 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
       const T v = C::load(st[off + xl]);
       H = (i == 0) ? v : H + v;
     });
-    return pseudo_potential<Q, T, kPsiKind, kFastExp>(a.phys, rho_of(H));
+    return pseudo_potential<Q, T, kPsiKind, kFastExp>(a.phys, PairRho<S>::of(a.phys, H));
   };
 
   // The thread's columns lie in one 32-column flag chunk.
@@ -690,18 +519,7 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
         if constexpr (kRegs) fnext[p][i] = v;
         H = (i == 0) ? v : H + v;
       });
-      const F2 rho = rho_of2(H);
-      float2 psi2;
-      if constexpr (kPsiKind == 0 && kFastExp) {
-        // psi_exp_fast of both nodes, the product and the fused
-        // multiply-add packed
-        const F2 e2 = rho * F2::splat(a.phys.exp2_scale);
-        psi2 = fma2(F2(ex2_approx(e2.x()), ex2_approx(e2.y())), F2::splat(-a.phys.rho0),
-                    F2::splat(a.phys.rho0)).v;
-      } else {
-        psi2 = make_float2(pseudo_potential<Q, T, kPsiKind, kFastExp>(a.phys, rho.x()),
-                           pseudo_potential<Q, T, kPsiKind, kFastExp>(a.phys, rho.y()));
-      }
+      const float2 psi2 = pair_psi<Q, S, FL>(a.phys, PairRho<S>::of(a.phys, H));
       *reinterpret_cast<float2*>(ring_row + RO + xa + 2 * p) = psi2;
       if constexpr (kRegs) rho_next[p] = H;
     }
@@ -740,285 +558,11 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
       }
 #pragma unroll
       for (int p = 0; p < P; ++p) {
-        const int xp = x + 2 * p;           // first column of pair p
-        const bool pair_ok = xp + 1 < a.nx;  // both nodes exist
-        // f_: the stored values (f, or h = sigma (f - w rho_s) for 16-bit
-        // storage).  H: their sum in table order (the psi pass's sum), rho
-        // from it; J = sum f_i c_i (D2Q9: the diagonal differences f5 - f7
-        // and f8 - f6 shared by its two components; otherwise in table
-        // order), j = J / sigma (the shifts carry no momentum).
-        F2 (&f_)[Q] = f[p];
-        const F2 Hm = rho_cur[p];
-        const F2 rho = rho_of2(Hm);
-        F2 Jx, Jy;
-        if constexpr (Q == 9) {
-          const F2 d57 = f_[5] - f_[7], d86 = f_[8] - f_[6];
-          Jx = ((f_[1] - f_[3]) + d57) + d86;
-          Jy = ((f_[2] - f_[4]) + d57) - d86;
-        } else {
-          Jx = F2::splat(0.f);
-          Jy = F2::splat(0.f);
-          static_for<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            if constexpr (L::cx(i) != 0) Jx = fma2(f_[i], F2::splat(T(L::cx(i))), Jx);
-            if constexpr (L::cy(i) != 0) Jy = fma2(f_[i], F2::splat(T(L::cy(i))), Jy);
-          });
-        }
-        F2 jx = Jx, jy = Jy;
-        if constexpr (C::kShifted && C::kScale != 1.0f) {
-          jx = Jx * F2::splat(kInvScale);
-          jy = Jy * F2::splat(kInvScale);
-        }
-        const F2 inv_rho(rcp_node<S, float>(rho.x()), rcp_node<S, float>(rho.y()));
-        const F2 ux = jx * inv_rho;
-        const F2 uy = jy * inv_rho;
-
-        // Neighbour psi, sum_i w_i psi(x + c_i) c_i.
-        F2 sfx = F2::splat(0.f), sfy = F2::splat(0.f), psi_c;
-        if constexpr (Q != 9) {
-          // Ring row of node row yo + c_y; the psi pair at column offset c_x
-          // is one aligned pair (c_x even) or the halves of two.
-          auto ring_at = [&](int cy, int o) -> float2 {
-            return *reinterpret_cast<const float2*>(
-                ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + RO + xa + 2 * p + o);
-          };
-          psi_c = F2(ring_at(0, 0));
-          static_for<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr int cx = L::cx(i), cy = L::cy(i);
-            if constexpr (i == L::REST) return;
-            F2 nb;
-            if constexpr ((cx & 1) == 0) {
-              nb = F2(ring_at(cy, cx));
-            } else {
-              nb = F2(ring_at(cy, cx - 1).y, ring_at(cy, cx + 1).x);
-            }
-            if constexpr (cx != 0) sfx = fma2(nb, F2::splat(T(L::w(i) * cx)), sfx);
-            if constexpr (cy != 0) sfy = fma2(nb, F2::splat(T(L::w(i) * cy)), sfy);
-          });
-        } else {
-          // D2Q9: three aligned pairs per ring row cover the pair's columns
-          // and one more on either side.
-          static_for<0, 3>([&](auto rc) {
-            constexpr int cy = decltype(rc)::value - 1;
-            const T* row = ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + RO + xa + 2 * p;
-            const float2 A = *reinterpret_cast<const float2*>(row - 2);
-            const float2 B = *reinterpret_cast<const float2*>(row);
-            const float2 Cc = *reinterpret_cast<const float2*>(row + 2);
-            const F2 pm(A.y, B.x), p0(B), pp(B.y, Cc.x);   // psi at c_x = -1, 0, +1
-            if constexpr (cy == 0) {
-              psi_c = p0;
-              sfx = fma2(pp - pm, F2::splat(T(L::w(1))), sfx);  // (1,0) and (-1,0)
-            } else {
-              // (0,cy): weight w_axis; (+-1, cy): weight w_diag
-              constexpr T sg = cy > 0 ? T(1) : T(-1);
-              sfy = fma2(p0, F2::splat(sg * T(L::w(2))), sfy);
-              sfy = fma2(pp + pm, F2::splat(sg * T(L::w(5))), sfy);
-              sfx = fma2(pp - pm, F2::splat(T(L::w(5))), sfx);
-            }
-          });
-        }
-
-        // Force: F_FF, then the wall terms on flagged chunks, then body force.
-        const F2 mg = F2::splat(-a.phys.G) * psi_c;
-        F2 Fx, Fy;
-        if (flag != 0u) {
-          const F2 ffx = mg * sfx, ffy = mg * sfy;
-          T phe[2] = {0, 0}, Sx[2] = {0, 0}, Sy[2] = {0, 0}, wx[2] = {0, 0}, wy[2] = {0, 0};
-  #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            if (xp + e < a.nx) {
-              const int64_t n = (int64_t)yo * a.nx + xp + e;
-              phe[e] = a.wall.phie[n];
-              Sx[e] = a.wall.sx[n];
-              Sy[e] = a.wall.sy[n];
-              if (a.wall.uwx) {
-                wx[e] = a.wall.uwx[n];
-                wy[e] = a.wall.uwy[n];
-              }
-            }
-          }
-          const F2 rp = rho * F2(phe[0], phe[1]);
-          const F2 dfx = rp * (F2(wx[0], wx[1]) - ux - ffx * inv_rho);
-          const F2 dfy = rp * (F2(wy[0], wy[1]) - uy - ffy * inv_rho);
-          Fx = ((ffx + rho * F2(Sx[0], Sx[1])) + dfx) + F2::splat(a.phys.bfx);
-          Fy = ((ffy + rho * F2(Sy[0], Sy[1])) + dfy) + F2::splat(a.phys.bfy);
-        } else {
-          Fx = fma2(mg, sfx, F2::splat(a.phys.bfx));
-          Fy = fma2(mg, sfy, F2::splat(a.phys.bfy));
-        }
-
-        if (xp < a.nx) {
-          if (!(fabsf(rho.x()) <= 3.0e38f) || (pair_ok && !(fabsf(rho.y()) <= 3.0e38f)))
-            atomicOr(a.status, kStatusNonFinite);
-          if constexpr (MODE == kModeStep) {
-            const F2 usx = fma2(Fx, inv_rho, ux);
-            const F2 usy = fma2(Fy, inv_rho, uy);
-            // EDM-BGK in pair form (see node_collide), packed over the two nodes
-            // and written as fused multiply-adds: with ca = c.(u* - g u) / theta
-            // and sb = omega - B + ((c.u*)^2 - g (c.u)^2) / (2 theta^2),
-            // f_post(+-c) = g f(+-c) + w rho (sb +- ca).
-            const F2 gg = F2::splat(a.phys.one_m_omega), ngg = F2::splat(-a.phys.one_m_omega);
-            const F2 ax3 = fma2(ngg, ux, usx) * F2::splat(T(E::inv_theta));
-            const F2 ay3 = fma2(ngg, uy, usy) * F2::splat(T(E::inv_theta));
-            const F2 us2 = fma2(usy, usy, usx * usx), u2 = fma2(uy, uy, ux * ux);
-            const F2 wB = fma2(fma2(ngg, u2, us2), F2::splat(-T(E::inv_2theta)),
-                               F2::splat(a.phys.omega));
-            if (FL != kFlExpPlain && a.phys.project) {
-              // rare path: per node.  The projection is linear and maps the
-              // shift w_i rho_s to itself, so it acts on h with (H, J) as it
-              // acts on f with (rho, j).
-              T fa[Q], fb[Q];
-  #pragma unroll
-              for (int i = 0; i < Q; ++i) {
-                fa[i] = f_[i].x();
-                fb[i] = f_[i].y();
-              }
-              project<Q, T>(fa, Hm.x(), Jx.x(), Jy.x());
-              project<Q, T>(fb, Hm.y(), Jx.y(), Jy.y());
-  #pragma unroll
-              for (int i = 0; i < Q; ++i) f_[i] = F2(fa[i], fb[i]);
-            }
-            if constexpr (C::kShifted) {
-              // The same update on h = sigma (f - w rho_s):
-              //   h_post(+-c) = g h(+-c) + sigma w [rho (sb +- ca) - omega rho_s].
-              const F2 nwr = F2::splat(a.phys.neg_omega_rho_s);
-              static_for<0, Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                constexpr int j = opposite<Q>(i);
-                if constexpr (i != L::REST && i < j) {
-                  const F2 cs = cdot2<L::cx(i), L::cy(i)>(usx, usy);
-                  const F2 cu = cdot2<L::cx(i), L::cy(i)>(ux, uy);
-                  const F2 ca = cdot2<L::cx(i), L::cy(i)>(ax3, ay3);
-                  const F2 t = fma2(ngg, cu * cu, cs * cs);
-                  const F2 sb = fma2(t, F2::splat(T(E::inv_2theta2)), wB);
-                  const F2 z = fma2(rho, sb, nwr);
-                  const F2 sw = F2::splat(T(C::kScale * L::w(i)));
-                  const F2 hi = fma2(gg, f_[i], sw * fma2(rho, ca, z));
-                  const F2 hj = fma2(gg, f_[j], sw * fma2(rho, -ca, z));
-                  f_[i] = hi;
-                  f_[j] = hj;
-                }
-              });
-            } else {
-              static_for<0, Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                constexpr int j = opposite<Q>(i);
-                // The rest population comes from the mass closure below.
-                if constexpr (i != L::REST && i < j) {
-                  const F2 cs = cdot2<L::cx(i), L::cy(i)>(usx, usy);
-                  const F2 cu = cdot2<L::cx(i), L::cy(i)>(ux, uy);
-                  const F2 ca = cdot2<L::cx(i), L::cy(i)>(ax3, ay3);
-                  const F2 wr = F2::splat(T(L::w(i))) * rho;
-                  const F2 t = fma2(ngg, cu * cu, cs * cs);
-                  const F2 sb = fma2(t, F2::splat(T(E::inv_2theta2)), wB);
-                  const F2 fi = fma2(gg, f_[i], wr * (sb + ca));
-                  const F2 fj = fma2(gg, f_[j], wr * (sb - ca));
-                  f_[i] = fi;
-                  f_[j] = fj;
-                }
-              });
-            }
-            {  // mass closure of the rest population: the stored values sum to
-               // H (rho, or sigma (rho - rho_s) for 16-bit storage) after the
-               // collision as before it
-              constexpr int i0 = L::REST == 0 ? 1 : 0;
-              F2 moving = f_[i0];
-#pragma unroll
-              for (int i = i0 + 1; i < Q; ++i)
-                if (i != L::REST) moving += f_[i];
-              f_[L::REST] = Hm - moving;
-            }
-            // Round both nodes once (stochastic rounding: bits from the node
-            // pair and the step), then the primary store plus periodic images.
-            typename PR::Raw raw[Q];
-            if constexpr (C::kShifted) {
-              if (FL == kFlExpPlain || a.stochastic) {
-                const uint32_t h = sr_hash((uint32_t)xp, (uint32_t)yo, key);
-                static_for<0, Q>([&](auto ic) {
-                  constexpr int i = decltype(ic)::value;
-                  raw[i] = PR::store_sr(f_[i], h * sr_multiplier(i));
-                });
-              } else {
-  #pragma unroll
-                for (int i = 0; i < Q; ++i) raw[i] = PR::store_rn(f_[i]);
-              }
-            } else {
-  #pragma unroll
-              for (int i = 0; i < Q; ++i) raw[i] = PR::store_rn(f_[i]);
-            }
-            S* out = a.fout + (int64_t)(yo + GY) * a.pitch + xp + GX;
-            if (pair_ok) {
-              static_for<0, Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                *reinterpret_cast<typename PR::Raw*>(out + Planes<Q>::template plane<i> * a.plane) =
-                    raw[i];
-              });
-            } else {
-              static_for<0, Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                out[Planes<Q>::template plane<i> * a.plane] = PR::lane(raw[i], 0);
-              });
-            }
-            const bool xedge = strip_edge && (xp < GX || xp + 1 >= a.nx - GX);
-            const bool yedge = yo < GY || yo >= a.ny - GY;
-            if ((xedge || yedge) && pair_ok && simple_images) {
-              // Both nodes of the pair have the same images: at most one
-              // column shift (+-nx) and one row shift (+-ny), stored as pairs.
-              const int sx = !xedge ? 0 : (xp < GX ? a.nx : -a.nx);
-              const int64_t sy = !yedge ? 0 : (int64_t)(yo < GY ? a.ny : -a.ny) * a.pitch;
-              auto put = [&](int64_t d) {
-                static_for<0, Q>([&](auto ic) {
-                  constexpr int i = decltype(ic)::value;
-                  *reinterpret_cast<typename PR::Raw*>(out + d + Planes<Q>::template plane<i> * a.plane) =
-                      raw[i];
-                });
-              };
-              if (sx != 0) put(sx);
-              if (sy != 0) {
-                put(sy);
-                if (sx != 0) put(sy + sx);
-              }
-            } else if (xedge || yedge) {
-  #pragma unroll 1
-              for (int e = 0; e < 2; ++e) {
-                const int xn = xp + e;
-                if (xn >= a.nx) break;
-                int xs = xn;
-                while (xs - a.nx >= -GX) xs -= a.nx;
-                int ya = yo;
-                while (ya - a.ny >= -GY) ya -= a.ny;
-                for (int ym = ya; ym < a.ny + GY; ym += a.ny) {
-                  for (int xm = xs; xm < a.nx + GX; xm += a.nx) {
-                    if (xm == xn && ym == yo) continue;
-                    S* o2 = a.fout + (int64_t)(ym + GY) * a.pitch + xm + GX;
-                    static_for<0, Q>([&](auto ic) {
-                      constexpr int i = decltype(ic)::value;
-                      o2[Planes<Q>::template plane<i> * a.plane] = PR::lane(raw[i], e);
-                    });
-                  }
-                }
-              }
-            }
-          } else {
-  #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              if (xp + e >= a.nx) break;
-              const int64_t n = (int64_t)yo * a.nx + xp + e;
-              const double r = e == 0 ? rho.x() : rho.y();
-              const double px = (double)(e == 0 ? jx.x() : jx.y()) + 0.5 * (double)(e == 0 ? Fx.x() : Fx.y());
-              const double py = (double)(e == 0 ? jy.x() : jy.y()) + 0.5 * (double)(e == 0 ? Fy.x() : Fy.y());
-              a.out_rho[n] = r;
-              if (a.momentum) {
-                a.out_ux[n] = px;
-                a.out_uy[n] = py;
-              } else {
-                a.out_ux[n] = px / r;
-                a.out_uy[n] = py / r;
-              }
-            }
-          }
-        }
+        pair_update<Q, S, kModeStep, FL>(
+            a, f[p], rho_cur[p], flag, x + 2 * p, yo, strip_edge, simple_images, key,
+            [&](int cy) -> const T* {  // ring row of node row yo + c_y
+              return ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + RO + xa + 2 * p;
+            });
       }  // pairs
     }
     if (++s == NS) {
@@ -1044,15 +588,15 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
 
 // Marches one segment with the variant the shape selects (one or two nodes
 // per thread).
-template <int Q, typename S, int W, int NS, int MODE, int FL, typename Args>
+template <int Q, typename S, int W, int NS, int FL, typename Args>
 __device__ __forceinline__ bool march_any(const PopMaps* src, const CUtensorMap* flg,
                                           const Args& a, int x0, int y0, int Lr, bool rev,
                                           const StepSmem<Q, S, W, NS>& sm, uint32_t& g,
                                           uint64_t policy) {
   if constexpr (StepShape<Q, S, W, NS>::V >= 2)
-    return march_segment_v2<Q, S, W, NS, MODE, FL>(src, flg, a, x0, y0, Lr, rev, sm, g);
+    return march_segment_v2<Q, S, W, NS, FL>(src, flg, a, x0, y0, Lr, rev, sm, g);
   else
-    return march_segment<Q, S, W, NS, MODE, FL>(src, flg, a, x0, y0, Lr, rev, sm, g, policy);
+    return march_segment<Q, S, W, NS, FL>(src, flg, a, x0, y0, Lr, rev, sm, g, policy);
 }
 
 // One time step of one lattice: CTA (bx, by) marches strip bx, segment by.
@@ -1060,7 +604,7 @@ __device__ __forceinline__ bool march_any(const PopMaps* src, const CUtensorMap*
 // at about the same time, pull the rows they share (the 2R halo rows of their
 // common edge) both at their start or both at their end: the second pull of
 // such a row is an L2 hit instead of a DRAM read.
-template <int Q, typename S, int W, int NS, int MODE, int MINB, int FL>
+template <int Q, typename S, int W, int NS, int MINB, int FL>
 __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
     step_kernel(const __grid_constant__ PopMaps src, const __grid_constant__ CUtensorMap flg,
                 const StepArgs<typename Codec<S>::T, S> a) {
@@ -1077,8 +621,8 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
   griddep_wait();
   // Every CTA reads the counter in march_any before this launch ends; the
   // word written here is read only by the next step.
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<MODE>(a);
-  march_any<Q, S, W, NS, MODE, FL>(&src, &flg, a, blockIdx.x * W, y0, min(a.tile_rows, a.ny - y0),
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<kModeStep>(a);
+  march_any<Q, S, W, NS, FL>(&src, &flg, a, blockIdx.x * W, y0, min(a.tile_rows, a.ny - y0),
                                (blockIdx.y & 1u) != 0u, sm, g, policy);
 }
 
@@ -1142,7 +686,7 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
     const int y1 = (int)((int64_t)a.ny * (seg + 1) / P.nseg[m]);
     if (threadIdx.x == 0 && local == 0) advance_key<kModeStep>(a);
     const auto* mb = &members[m];
-    return march_any<Q, S, W, NS, kModeStep, FL>(&mb->map[dir], &mb->flags, a, x0, y0, y1 - y0,
+    return march_any<Q, S, W, NS, FL>(&mb->map[dir], &mb->flags, a, x0, y0, y1 - y0,
                                                 (seg & 1) != 0, sm, g, policy);
   };
   if constexpr (PERSIST) {

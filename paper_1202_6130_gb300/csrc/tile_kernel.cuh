@@ -1,0 +1,322 @@
+// The fused time step on two-dimensional tiles: a CTA updates TW x TH nodes at
+// once, for TS time steps, instead of marching row by row (step_kernel.cuh).
+//
+// What bounds a march on small and middle lattices is its serial chain: about
+// 0.9 us per row (stage wait, psi, barrier, collision), with too few strips and
+// segments to fill the chip.  A tile does all its rows at once: one load of
+// everything it reads, psi of the tile and its halo, one barrier, the
+// collision.  GB300, us per step, march -> tiles: D2Q9 128x64 FP32 6.4 -> 3.0 and
+// FP64 40.6 -> 9.9, 400x200 FP32 7.9 -> 4.3, 1024x512 FP16S 9.2 -> 6.7, D2Q21
+// 650x150 FP32 10.8 -> 6.4.  Tiles also need a quarter fewer instructions per
+// node (no ring or stage bookkeeping per row: 5.8 warp instructions against 8.2
+// on 2048x1024 FP16S) and, for D2Q21, no second read of the row from its stage
+// with four stages pinned: D2Q21 4096x2048 FP32 314 -> 256 and FP16S 175 -> 155;
+// FP64 2048x1024 726 -> 637.  Tiles that touch no edge and no wall run a second
+// copy of the update without that code (IN): 63.3 against 65.4 us on 4096x2048
+// FP16S; on small lattices, where every tile has an edge, it only costs.
+#pragma once
+
+#include "node_update.cuh"
+#include "tma.cuh"
+
+namespace lbm {
+
+// Shape and shared-memory layout of a tile CTA.
+//
+// The populations that the tile's TS steps read arrive as one TMA box per plane
+// group (the planes with one c_y): BW columns (the tile and GX ghost columns on
+// either side, so that the box starts on 16 bytes) by BH rows.  Row b of a
+// group's box is the source row of node row y0 - BR + b, so a node pulls every
+// population from the same box row.  Step s updates the tile and margin(s)
+// nodes around it, which is what the later steps still read; nodes around the
+// tile are other tiles' nodes (or their periodic images), recomputed with the
+// same arithmetic.  Post-collision values go back into the boxes, to the place
+// the next step pulls them from.
+template <int Q_, typename S_, int TW_, int TH_, int NT_, int TS_, bool IN_> struct TileShape {
+  using S = S_;
+  using L = Lattice<Q_>;
+  using P = Planes<Q_>;
+  using T = typename Codec<S>::T;
+  static constexpr int Q = Q_, R = L::R, TW = TW_, TH = TH_, NT = NT_, TS = TS_;
+  static constexpr bool IN = IN_;  // a second copy of the update without edge and wall code
+  static constexpr int GX = ghost_x<S, R>(), GY = ghost_y<R>();
+  static constexpr int V = (sizeof(T) == 4 && (Q == 9 || sizeof(S) == 2)) ? 2 : 1;  // as StepShape
+  static constexpr int margin(int s) { return 2 * R * (TS - 1 - s); }
+  static constexpr int BR = R + margin(0);
+  static constexpr int BW = TW + 2 * GX, BH = TH + 2 * BR;
+  static constexpr int NBOX = 2 * R + 1;
+  // Work items (node pairs, or nodes) of step s: prow(s) per row, over the
+  // tile and its margin; slots(s) of them per thread.
+  static constexpr int prow(int s) { return (TW + 2 * margin(s)) / V; }
+  static constexpr int items(int s) { return prow(s) * (TH + 2 * margin(s)); }
+  static constexpr int slots(int s) { return (items(s) + NT - 1) / NT; }
+  // psi: RO columns and BR rows around the tile (RO even for pairs).
+  static constexpr int RP = V == 2 ? (R + 1) / 2 * 2 : R;
+  static constexpr int RO = margin(0) + RP;
+  static constexpr int PW = TW + 2 * RO;
+  // The psi columns beside the updated nodes are formed as whole items where
+  // the boxes hold what their outer nodes pull, else node by node.
+  static constexpr bool kHaloItems = RO + R <= GX;
+  static constexpr uint32_t TX = Q * BW * BH * (uint32_t)sizeof(S);
+  struct Tables {
+    int pop[Q];  // element offset of population i of node column -GX, row -BR
+    int box_cy[NBOX], box_plane[NBOX], box_depth[NBOX], box_off[NBOX], box_map[NBOX];
+    int depth[kMaxMaps];
+    int nmap, bytes;
+  };
+  static constexpr Tables make() {
+    Tables t{};
+    int off = 0;
+    for (int j = 0; j < NBOX; ++j) {
+      const int cy = j - R;
+      int first = Q, n = 0;
+      for (int i = 0; i < Q; ++i) {
+        if (L::cy(i) != cy) continue;
+        ++n;
+        if (P::kTable.plane[i] < first) first = P::kTable.plane[i];
+      }
+      t.box_cy[j] = cy;
+      t.box_plane[j] = first;
+      t.box_depth[j] = n;
+      t.box_off[j] = off;
+      int k = 0;
+      while (k < t.nmap && t.depth[k] != n) ++k;
+      if (k == t.nmap) t.depth[t.nmap++] = n;
+      t.box_map[j] = k;
+      off += (n * BW * BH * (int)sizeof(S) + 127) / 128 * 128;
+    }
+    t.bytes = off;
+    for (int i = 0; i < Q; ++i) {
+      const int j = L::cy(i) + R;
+      t.pop[i] = t.box_off[j] / (int)sizeof(S) + (P::kTable.plane[i] - t.box_plane[j]) * BW * BH;
+    }
+    return t;
+  }
+  static constexpr Tables kTab = make();
+  static constexpr int NMAP = kTab.nmap;
+  static constexpr int SMEM = 128 /*alignment slack*/ + kTab.bytes + PW * BH * (int)sizeof(T) + 16;
+  static_assert(TW % 16 == 0 && NT % 32 == 0, "tile shape");
+  static_assert(BW <= 256 && BH <= 256 && NMAP <= kMaxMaps, "tensor-map boxes");
+  static_assert(margin(0) + 2 * R <= GX && margin(0) + 2 * R <= GY, "ghost frame");
+  static_assert(TS == 1 || (TS % 2 == 0 && V == 2 && R == 1), "several steps: D2Q9 node pairs");
+  static_assert(kHaloItems || R == 1, "halo columns node by node: R = 1");
+};
+
+// Advances the tile with origin (x0, y0) by TS time steps (kModeStep), or writes
+// its moments (kModeMoments, TS = 1).
+template <typename Sh, int MODE, int FL, typename Args>
+__device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* __restrict__ flags,
+                                            int flag_pitch, const Args& a, int x0, int y0,
+                                            unsigned char* smem_raw) {
+  using S = typename Sh::S;
+  using T = typename Sh::T;
+  using C = Codec<S>;
+  using L = typename Sh::L;
+  constexpr int Q = Sh::Q, R = Sh::R, GX = Sh::GX, GY = Sh::GY, V = Sh::V, NT = Sh::NT;
+  constexpr int PW = Sh::PW, BW = Sh::BW, BR = Sh::BR, TS = Sh::TS;
+  unsigned char* const base = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
+  S* const st = reinterpret_cast<S*>(base);
+  constexpr int kPopBytes = Sh::kTab.bytes;
+  T* const psi = reinterpret_cast<T*>(base + kPopBytes);
+  uint64_t* const bar = reinterpret_cast<uint64_t*>(psi + PW * Sh::BH);
+  int* const s_abort = reinterpret_cast<int*>(bar + 1);
+  const int tid = threadIdx.x;
+
+  if (tid == 0) {
+    mbar_init(bar, 1);
+    *s_abort = 0;
+    fence_barrier_init();
+    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src->m[decltype(kc)::value]); });
+  }
+  // A programmatic dependent of the previous step (see step_kernel).
+  griddep_launch_dependents();
+  griddep_wait();
+  if (tid == 0) {
+    mbar_arrive_expect_tx(bar, Sh::TX + a.extra_tx);
+    static_for<0, Sh::NBOX>([&](auto jc) {
+      constexpr int j = decltype(jc)::value;
+      constexpr int cy = Sh::kTab.box_cy[j], off = Sh::kTab.box_off[j], map = Sh::kTab.box_map[j];
+      constexpr int plane = Sh::kTab.box_plane[j];
+      tma_load_3d(base + off, &src->m[map], bar, x0, y0 - BR - cy + GY, plane);
+    });
+  }
+  const uint32_t key = step_key<S, MODE, FL>(a);
+  const bool simple_images = a.nx >= 2 * GX && a.ny >= 2 * GY && (V == 1 || (a.nx & 1) == 0);
+  __syncthreads();  // the barrier is initialised
+
+  // Address of population i as the node at (c, r) of the tile pulls it.
+  auto pop = [&](auto ic, int c, int r) -> S* {
+    constexpr int off = Sh::kTab.pop[decltype(ic)::value] + GX - L::cx(decltype(ic)::value);
+    return st + (off + (r + BR) * BW + c);
+  };
+  auto psi_at = [&](int c, int r) -> T* { return psi + (r + BR) * PW + Sh::RO + c; };
+  // psi of one node from its populations.
+  auto node_psi = [&](int c, int r) {
+    T H;
+    static_for<0, Q>([&](auto ic) {
+      const T v = C::load(*pop(ic, c, r));
+      H = (decltype(ic)::value == 0) ? v : H + v;
+    });
+    if constexpr (V == 2)
+      *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1, C::kShifted>(
+          a.phys, PairRho<S>::of(a.phys, H));
+    else
+      *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1>(a.phys, H);
+  };
+  // Loads the item at (c, r) (a node pair or a node) into f, its sum into H,
+  // and forms its psi.
+  using F = std::conditional_t<V == 2, F2, T>;
+  auto item_psi = [&](int c, int r, F (&f)[Q], F& H) {
+    static_for<0, Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      const S* p = pop(ic, c, r);
+      if constexpr (V == 1) {
+        f[i] = C::load(*p);
+      } else if constexpr ((L::cx(i) & 1) == 0) {
+        f[i] = Pair<S>::load(*reinterpret_cast<const typename Pair<S>::Raw*>(p));
+      } else {
+        f[i] = Pair<S>::load1(p[0], p[1]);
+      }
+      H = (i == 0) ? f[i] : H + f[i];
+    });
+    if constexpr (V == 2)
+      *reinterpret_cast<float2*>(psi_at(c, r)) =
+          pair_psi<Q, S, FL>(a.phys, PairRho<S>::of(a.phys, H));
+    else
+      *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1>(a.phys, H);
+  };
+  auto wrap_x = [&](int x) { return x < 0 ? x + a.nx : (x >= a.nx ? x - a.nx : x); };
+  auto wrap_y = [&](int y) { return y < 0 ? y + a.ny : (y >= a.ny ? y - a.ny : y); };
+
+  const bool strip_edge = x0 < GX || x0 + Sh::TW > a.nx - GX;
+  bool aborted = false;
+  static_for<0, TS>([&](auto sc) {
+    constexpr int s = decltype(sc)::value;
+    constexpr int M = Sh::margin(s), SL = Sh::slots(s), PROW = Sh::prow(s), NI = Sh::items(s);
+    F f[SL][Q], H[SL];
+    int col[SL], row[SL];
+    uint32_t flag[SL];
+    bool on[SL];
+#pragma unroll
+    for (int k = 0; k < SL; ++k) {
+      if constexpr (NT % PROW == 0) {  // every slot in the thread's first column
+        row[k] = tid / PROW + k * (NT / PROW) - M;
+        col[k] = V * (tid % PROW) - M;
+      } else {
+        const int p = tid + k * NT, q = p / PROW;
+        row[k] = q - M;
+        col[k] = V * (p - q * PROW) - M;
+      }
+      const int x = x0 + col[k], y = y0 + row[k];
+      on[k] = (NI % NT == 0 || tid + k * NT < NI) && x < a.nx + M && y < a.ny + M;
+      const int xw = M ? wrap_x(x) : x, yw = M ? wrap_y(y) : y;
+      flag[k] = a.wall.active && on[k] ? flags[(int64_t)yw * flag_pitch + (xw >> 5)] : 0u;
+    }
+    if constexpr (s == 0) {
+      if (!mbar_wait_bounded(bar, 0, a.wait_ns)) *s_abort = 1;
+    } else {
+      __syncthreads();  // the previous step's populations are in place, its psi read
+    }
+#pragma unroll
+    for (int k = 0; k < SL; ++k)
+      if (NI % NT == 0 || tid + k * NT < NI) item_psi(col[k], row[k], f[k], H[k]);
+    // psi of the rows above and below the updated nodes, then of the columns
+    // on either side.
+    constexpr int HP = Sh::kHaloItems ? PROW + 2 * Sh::RP / V : PROW;
+    constexpr int HC = Sh::kHaloItems ? 2 * Sh::RP / V * (Sh::TH + 2 * M) : 0;
+    for (int h = tid; h < 2 * R * HP + HC; h += NT) {
+      int c, r;
+      if (HC == 0 || h < 2 * R * HP) {
+        const int q = h / HP;
+        c = V * (h - q * HP) - M - (Sh::kHaloItems ? Sh::RP : 0);
+        r = q < R ? q - R - M : Sh::TH + M + q - R;
+      } else {
+        constexpr int HR = Sh::TH + 2 * M;
+        const int q = (h - 2 * R * HP) / HR;
+        c = q < Sh::RP / V ? V * q - Sh::RP - M : Sh::TW + M + V * (q - Sh::RP / V);
+        r = h - 2 * R * HP - q * HR - M;
+      }
+      F fh[Q], Hh;
+      item_psi(c, r, fh, Hh);
+    }
+    if constexpr (!Sh::kHaloItems) {
+      constexpr int NR = Sh::TH + 2 * M + 2;
+      for (int h = NT - 1 - tid; h < 2 * NR; h += NT)
+        node_psi(h < NR ? -M - 1 : Sh::TW + M, (h < NR ? h : h - NR) - M - 1);
+    }
+    uint32_t any = 0;
+    if constexpr (Sh::IN) {
+#pragma unroll
+      for (int k = 0; k < SL; ++k) any |= flag[k];
+      any = __syncthreads_or((int)any);
+    } else {
+      __syncthreads();
+    }
+    // psi is complete; every population has been read.
+    aborted = *s_abort != 0;
+    if (aborted) return;
+    auto collide = [&](auto ec) {
+      constexpr bool E = decltype(ec)::value;
+#pragma unroll
+      for (int k = 0; k < SL; ++k) {
+        if (E ? !on[k] : !(NI % NT == 0 || tid + k * NT < NI)) continue;
+        const int x = x0 + col[k], y = y0 + row[k];
+        auto psi_row = [&](int cy) -> const T* { return psi_at(col[k], row[k] + cy); };
+        if constexpr (V == 1) {
+          node_update<Q, S, MODE, FL, E>(a, f[k], flag[k], x, y, strip_edge, simple_images, psi_row);
+        } else if constexpr (s == TS - 1) {
+          pair_update<Q, S, MODE, FL, E>(a, f[k], H[k], flag[k], x, y, strip_edge, simple_images,
+                                      key + (uint32_t)s, psi_row);
+        } else {
+          // Even nx: the pair and its periodic images are pairs of whole nodes.
+          const int xw = E ? wrap_x(x) : x, yw = E ? wrap_y(y) : y;
+          PairAt at;
+          at.n0 = (int64_t)yw * a.nx + xw;
+          at.n1 = at.n0 + 1;
+          at.ok0 = at.ok1 = true;
+          at.hx = (uint32_t)xw;
+          at.hy = (uint32_t)yw;
+          const PairState<Q, S, E> n(a, f[k], H[k], flag[k], at, psi_row);
+          typename Pair<S>::Raw raw[Q];
+          pair_collide<Q, S, FL>(a, n, f[k], H[k], at, key + (uint32_t)s, raw);
+          static_for<0, Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            constexpr int off = Sh::kTab.pop[i] + GX;
+            *reinterpret_cast<typename Pair<S>::Raw*>(
+                st + (off + (row[k] + L::cy(i) + BR) * BW + col[k])) = raw[i];
+          });
+        }
+      }
+    };
+    const bool inside = Sh::IN && x0 >= GX && x0 + Sh::TW <= a.nx - GX && y0 >= GY && y0 + Sh::TH <= a.ny - GY && !any;
+    if constexpr (Sh::IN) {
+      if (inside) {
+        collide(std::false_type{});
+        return;
+      }
+    }
+    collide(std::true_type{});
+  });
+  if (aborted && tid == 0) {
+    // The boxes never arrived in full.  Record it, retire the bytes that the
+    // barrier was told to expect beyond its copies (the test hook), and wait
+    // (bounded) for the copies still in flight.
+    atomicOr(a.status, kStatusTimeout);
+    if (a.extra_tx) mbar_complete_tx(bar, a.extra_tx);
+    mbar_wait_bounded(bar, 0, a.wait_ns);
+  }
+}
+
+// TS time steps of one lattice; CTA (bx, by) updates the tile at (bx TW, by TH).
+template <typename Sh, int MODE, int FL, int MINB>
+__global__ void __launch_bounds__(Sh::NT, MINB)
+    tile_kernel(const __grid_constant__ PopMaps src, const uint32_t* __restrict__ flags,
+                int flag_pitch, const StepArgs<typename Sh::T, typename Sh::S> a) {
+  extern __shared__ unsigned char smem_raw[];
+  tile_update<Sh, MODE, FL>(&src, flags, flag_pitch, a, blockIdx.x * Sh::TW, blockIdx.y * Sh::TH,
+                            smem_raw);
+  if constexpr (MODE == kModeStep)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<MODE>(a, Sh::TS);
+}
+
+}  // namespace lbm

@@ -22,24 +22,21 @@ class TorchAllocator:
         import torch
         self.torch = torch
         self.device = torch.device(device)
-        self.stream = stream if isinstance(stream, torch.cuda.Stream) else None
-        self.live = {}
+        self.stream = stream  # None: the current stream
         self._alloc = L.ALLOC_FN(self._alloc_cb)
         self._free = L.FREE_FN(self._free_cb)
         self.struct = L.lbm_allocator(self._alloc, self._free, None)
 
     def _alloc_cb(self, nbytes, user):
+        cuda = self.torch.cuda
         try:
-            with self.torch.cuda.stream(self.stream):  # None: the current stream
-                t = self.torch.empty(int(nbytes), dtype=self.torch.uint8, device=self.device)
+            stream = self.stream if self.stream is not None else cuda.current_stream(self.device)
+            return cuda.caching_allocator_alloc(int(nbytes), self.device, stream.cuda_stream)
         except Exception:  # out of memory -> NULL -> LBM_ENOMEM
             return None
-        p = t.data_ptr()
-        self.live[p] = t
-        return p
 
     def _free_cb(self, ptr, user):
-        self.live.pop(ptr, None)
+        self.torch.cuda.caching_allocator_delete(ptr)
 
 
 def _c64(a, shape=None):

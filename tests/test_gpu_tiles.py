@@ -1,0 +1,77 @@
+"""The tile kernel against the row march: the same
+node arithmetic in other places, so the same bits.  tile_rows > 0 asks for the
+row march; tile_rows = 0 lets the engine choose, which on these sizes is a tile
+shape."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+    torch.cuda.set_device(0)
+    import paper_1202_6130_gb300 as p
+    p.load()
+    return p
+
+
+def _case(nx, ny, lattice=9):
+    w = W.droplet_on_wall(nx=nx, ny=ny, R=max(2.0, min(nx, ny) / 3.0), seed=nx + ny, noise_amp=1e-4,
+                          lattice=lattice, tau=0.8)
+    w.u_wall = np.zeros((2, ny, nx))
+    w.u_wall[0] = 0.01 * W.uniform(3, ny * nx, 0.0, 1.0).reshape(ny, nx)
+    w.u_wall[1] = -0.005
+    w.body_force = (1e-5, -2e-6)
+    w.epsilon = 1.3
+    return w
+
+
+def _run(pkg, w, storage, tile_rows, steps, **kw):
+    sim = pkg.Simulation.from_workload(w, storage=storage, tile_rows=tile_rows, **kw)
+    for n in steps:
+        sim.step(n)
+    f, clock = sim.populations(), sim.clock()
+    sim.close()
+    return f, clock
+
+
+# D2Q9: smaller than a halo, than a tile, one more and one less than tiles of 32
+# and 64 columns and 4, 8, 12 and 24 rows, odd widths (a
+# lone last column), and the sizes from which the larger shapes are chosen.
+D2Q9 = [(1, 1), (2, 3), (4, 4), (6, 5), (8, 256), (32, 8), (34, 9), (62, 7), (64, 12), (66, 13),
+        (67, 35), (130, 25), (254, 49), (512, 384), (1026, 515), (1537, 771), (2048, 1024)]
+
+
+@pytest.mark.parametrize("size", D2Q9, ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("storage", ["fp32", "fp16s", "bf16s"])
+def test_tiles_equal_the_row_march_bitwise(pkg, size, storage):
+    """Seven steps, then one and four more."""
+    w = _case(*size)
+    want, c0 = _run(pkg, w, storage, 3, (7, 1, 4))
+    got, c1 = _run(pkg, w, storage, 0, (7, 1, 4))
+    np.testing.assert_array_equal(got, want)
+    assert c0 == c1
+
+
+@pytest.mark.parametrize("kw", [dict(rounding="nearest"), dict(project=True)],
+                         ids=["nearest", "project"])
+@pytest.mark.parametrize("storage", ["fp32", "bf16s"])
+def test_tiles_equal_the_row_march_with_run_time_switches(pkg, storage, kw):
+    w = _case(130, 50)
+    for size in ((130, 50), (1026, 515)):
+        w = _case(*size)
+        np.testing.assert_array_equal(_run(pkg, w, storage, 0, (6,), **kw)[0],
+                                      _run(pkg, w, storage, 4, (6,), **kw)[0])
+
+
+@pytest.mark.parametrize("size", [(1, 1), (5, 2), (17, 9), (33, 29), (66, 17), (131, 40), (1026, 515)],
+                         ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("lattice,storage", [(9, "fp64"), (21, "fp64"), (21, "fp32"), (21, "fp16s"),
+                                             (21, "bf16s")])
+def test_one_step_tiles_equal_the_row_march_bitwise(pkg, lattice, storage, size):
+    w = _case(*size, lattice=lattice)
+    np.testing.assert_array_equal(_run(pkg, w, storage, 0, (3,))[0], _run(pkg, w, storage, 4, (3,))[0])
