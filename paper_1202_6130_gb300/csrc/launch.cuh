@@ -80,9 +80,11 @@ template <int Q, typename S> constexpr TileList tile_list() {
   else if constexpr (Q == 21)
     return {{{32, 4, 64, 1, false, 8, 4.1}, {64, 8, 128, 1, true, 4, 6.9}}, 2, 1};
   else if constexpr (sizeof(S) == 4)
-    return {{{32, 4, 64, 1, false, 8, 2.8}, {64, 8, 128, 1, true, 7, 6.4}}, 2, 0};
+    return {{{32, 4, 64, 1, false, 8, 2.8}, {64, 8, 128, 1, true, 7, 6.4}, {32, 4, 160, 2, false, 4, 3.05},
+             {32, 8, 224, 2, false, 3, 3.5}, {64, 12, 288, 2, true, 3, 6.8}, {64, 24, 320, 2, true, 2, 8.8}}, 6, 0};
   else
-    return {{{32, 4, 64, 1, false, 8, 2.5}, {64, 8, 128, 1, true, 7, 4.1}}, 2, 0};
+    return {{{32, 4, 64, 1, false, 8, 2.5}, {64, 8, 128, 1, true, 7, 4.1}, {32, 4, 160, 2, false, 4, 3.4},
+             {32, 8, 224, 2, false, 3, 3.2}, {64, 12, 288, 2, true, 3, 6.0}, {64, 24, 320, 2, true, 2, 7.6}}, 6, 0};
 }
 template <int Q, typename S, int K> struct TileConfig {
   static constexpr TileCfg kCfg = tile_list<Q, S>().t[K];

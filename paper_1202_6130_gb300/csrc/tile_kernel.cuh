@@ -14,6 +14,21 @@
 // FP64 2048x1024 726 -> 637.  Tiles that touch no edge and no wall run a second
 // copy of the update without that code (IN): 63.3 against 65.4 us on 4096x2048
 // FP16S; on small lattices, where every tile has an edge, it only costs.
+//
+// Two steps per launch (TS = 2, D2Q9 node pairs): the tile's populations stay in
+// shared memory between the steps, so a pair of steps costs one launch, one load
+// latency and one trip through HBM; the price is the first step on 2 more nodes
+// on every side (8x larger tiles for the lattices that can afford them).  GB300,
+// us per step, best one-step kernel -> two steps: 128x64 FP32 3.0 -> 2.1, 400x200
+// FP32 4.3 -> 2.9, 1024x512 FP32 8.3 -> 7.6, 4096x2048 FP32 96 -> 80 (its DRAM
+// traffic halves; what bounds it then is latency between barriers at 20 warps
+// per SM, 45% of issue slots), 8192x4096 FP32 368 -> 304.  16-bit storage is
+// bound by instruction issue on large lattices and stays at one step there.
+//
+// Tried and dropped: persistent CTAs that prefetch the next tile's boxes under
+// the last collision (loop-invariant values took the registers: 184-628 bytes
+// of spills, 1.3x slower with two steps; no gain with one step, which did not
+// spill).
 #pragma once
 
 #include "node_update.cuh"

@@ -1,4 +1,4 @@
-"""The tile kernel against the row march: the same
+"""The tile kernel (one and two steps per launch) against the row march: the same
 node arithmetic in other places, so the same bits.  tile_rows > 0 asks for the
 row march; tile_rows = 0 lets the engine choose, which on these sizes is a tile
 shape."""
@@ -40,7 +40,7 @@ def _run(pkg, w, storage, tile_rows, steps, **kw):
 
 
 # D2Q9: smaller than a halo, than a tile, one more and one less than tiles of 32
-# and 64 columns and 4, 8, 12 and 24 rows, odd widths (a
+# and 64 columns and 4, 8, 12 and 24 rows, odd widths (one step per launch, a
 # lone last column), and the sizes from which the larger shapes are chosen.
 D2Q9 = [(1, 1), (2, 3), (4, 4), (6, 5), (8, 256), (32, 8), (34, 9), (62, 7), (64, 12), (66, 13),
         (67, 35), (130, 25), (254, 49), (512, 384), (1026, 515), (1537, 771), (2048, 1024)]
@@ -49,7 +49,8 @@ D2Q9 = [(1, 1), (2, 3), (4, 4), (6, 5), (8, 256), (32, 8), (34, 9), (62, 7), (64
 @pytest.mark.parametrize("size", D2Q9, ids=lambda s: "x".join(map(str, s)))
 @pytest.mark.parametrize("storage", ["fp32", "fp16s", "bf16s"])
 def test_tiles_equal_the_row_march_bitwise(pkg, size, storage):
-    """Seven steps, then one and four more."""
+    """Seven steps (three launches of two and one of one, or seven of one), then
+    one and four more."""
     w = _case(*size)
     want, c0 = _run(pkg, w, storage, 3, (7, 1, 4))
     got, c1 = _run(pkg, w, storage, 0, (7, 1, 4))
@@ -75,3 +76,17 @@ def test_tiles_equal_the_row_march_with_run_time_switches(pkg, storage, kw):
 def test_one_step_tiles_equal_the_row_march_bitwise(pkg, lattice, storage, size):
     w = _case(*size, lattice=lattice)
     np.testing.assert_array_equal(_run(pkg, w, storage, 0, (3,))[0], _run(pkg, w, storage, 4, (3,))[0])
+
+
+def test_checks_fall_between_the_steps_of_two(pkg):
+    """check_every = 3 reports a non-finite density on the step it is due (the
+    state stays as after that step), although two steps fit one launch."""
+    w = _case(64, 32)
+    sim = pkg.Simulation.from_workload(w, storage="fp32", check_every=3)
+    f = sim.populations()
+    f[:, 10, 10] = np.nan
+    sim.set_populations(f)
+    with pytest.raises(pkg.LbmError) as ei:
+        sim.step(8)
+    assert "ENONFINITE" in str(ei.value) and sim.steps_done() == 3
+    sim.close()
