@@ -49,9 +49,13 @@ __device__ __forceinline__ void write_moments(const Args& a, int64_t n, T rho, T
   if (a.momentum) {
     a.out_ux[n] = (double)jx + 0.5 * (double)Fx;
     a.out_uy[n] = (double)jy + 0.5 * (double)Fy;
+  } else if constexpr (sizeof(T) == 4) {
+    const float rc = __frcp_rn(rho);
+    a.out_ux[n] = half_force_velocity(jx, Fx, rho, rc);
+    a.out_uy[n] = half_force_velocity(jy, Fy, rho, rc);
   } else {
-    a.out_ux[n] = ((double)jx + 0.5 * (double)Fx) / (double)rho;
-    a.out_uy[n] = ((double)jy + 0.5 * (double)Fy) / (double)rho;
+    a.out_ux[n] = (jx + 0.5 * Fx) / rho;
+    a.out_uy[n] = (jy + 0.5 * Fy) / rho;
   }
 }
 
