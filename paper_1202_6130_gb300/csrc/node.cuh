@@ -153,7 +153,7 @@ __device__ __forceinline__ uint32_t sr_hash(uint32_t x, uint32_t y, uint32_t ste
 template <typename S, int R> __host__ __device__ constexpr int ghost_x() {
   return ((2 * R * (int)sizeof(S) + 15) / 16) * 16 / (int)sizeof(S);
 }
-template <int R> __host__ __device__ constexpr int ghost_y() { return 2 * R; }
+template <int R> __host__ __device__ constexpr int ghost_y() { return R == 1 ? 4 : 2 * R; }
 
 // ---------------------------------------------------------------------------
 // Run-time parameters of the update (compute precision T).
@@ -187,8 +187,8 @@ template <typename T> struct WallFields {
 template <typename T> __device__ __forceinline__ T t_exp(T v);
 template <> __device__ __forceinline__ double t_exp<double>(double v) { return exp(v); }
 template <> __device__ __forceinline__ float t_exp<float>(float v) { return expf(v); }
-// 1 / rho.  FP64 divides exactly (quotients then divide, like the oracle);
-// FP32 arithmetic: the hardware reciprocal (PTX rcp.approx.ftz.f32, at most
+// 1 / rho.  FP64: the correctly rounded reciprocal (div_rho forms quotients from
+// it); FP32 arithmetic: the hardware reciprocal (PTX rcp.approx.ftz.f32, at most
 // 1 ulp from the correctly rounded value).
 template <typename T> __device__ __forceinline__ T t_rcp(T v);
 template <> __device__ __forceinline__ double t_rcp<double>(double v) { return 1.0 / v; }
@@ -219,6 +219,23 @@ template <typename T> __device__ __forceinline__ T t_sqrt(T v);
 template <> __device__ __forceinline__ double t_sqrt<double>(double v) { return sqrt(v); }
 template <> __device__ __forceinline__ float t_sqrt<float>(float v) { return sqrtf(v); }
 
+// a / b from y = 1 / b, computed once per node.  FP64: the quotient a y corrected
+// by its exact remainder, which is the correctly rounded a / b when y is the
+// correctly rounded reciprocal (P. W. Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990), for 3 fused
+// operations instead of a division's dozen: the FP64 pipe bounds FP64 storage
+// (with the fused collision and neighbour sums, 2048x1024 D2Q9 637 -> 516 us
+// per step, 128x64 9.9 -> 8.4).
+// FP32 multiplies by y.
+template <typename T> __device__ __forceinline__ T div_rho(T a, T b, T y);
+template <> __device__ __forceinline__ double div_rho<double>(double a, double b, double y) {
+  const double q = a * y;
+  return fma(fma(-q, b, a), y, q);
+}
+template <> __device__ __forceinline__ float div_rho<float>(float a, float, float y) {
+  return a * y;
+}
+
 // 2^x by the hardware base-2 exponential (PTX ex2.approx.ftz.f32: a few
 // units in the last place over the range used here).
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -245,10 +262,13 @@ template <int Q, typename T, int KIND = -1, bool FAST = false>
 __device__ __forceinline__ T pseudo_potential(const Physics<T>& P, T rho) {
   if (KIND == 0 || (KIND < 0 && P.psi_kind == 0)) {
     if constexpr (FAST && sizeof(T) == 4) return psi_exp_fast(rho, P.exp2_scale, P.rho0);
-    // FP64 divides like the oracle; FP32 multiplies by the reciprocal (exact
-    // for the usual rho0 = 1).
-    const T arg = sizeof(T) == 8 ? -rho / P.rho0 : -rho * P.inv_rho0;
-    return P.rho0 * (T(1) - t_exp<T>(arg));
+    // FP64 divides (div_rho: the correctly rounded quotient); FP32 multiplies by
+    // the reciprocal (exact for the usual rho0 = 1).
+    if constexpr (sizeof(T) == 8) {
+      const T arg = P.rho0 == T(1) ? -rho : div_rho<T>(-rho, P.rho0, P.inv_rho0);
+      return P.rho0 * (T(1) - t_exp<T>(arg));
+    }
+    return P.rho0 * (T(1) - t_exp<T>(-rho * P.inv_rho0));
   }
   constexpr T theta = T(Lattice<Q>::THETA);
   T p;
@@ -336,16 +356,6 @@ __device__ __forceinline__ void project(T (&f)[Q], T rho, T jx, T jy) {
 }
 
 
-// a / b: FP64 divides (the oracle's rounding); FP32 multiplies by a reciprocal
-// computed once per node.
-template <typename T> __device__ __forceinline__ T div_rho(T a, T b, T inv_b);
-template <> __device__ __forceinline__ double div_rho<double>(double a, double b, double) {
-  return a / b;
-}
-template <> __device__ __forceinline__ float div_rho<float>(float a, float, float inv_b) {
-  return a * inv_b;
-}
-
 // v as FP64 by moving its bits (subnormal values become zero), on the integer
 // pipe: FP64 conversions share the FP64 pipe's 1/64 rate.
 __device__ __forceinline__ double f64_from_f32(float v) {
@@ -360,8 +370,8 @@ __device__ __forceinline__ double f64_from_f32(float v) {
 // two-sum) and the quotient into three: each is the leading FP32 quotient of
 // the remainder before it, the remainders being exact by a fused multiply-add
 // (a long division by words).  Their FP64 sum is the only FP64 work: two
-// additions instead of a division's dozen (the read-out of
-// 4096x2048 FP32: 367 -> 99 us, of BF16S 530 -> 90, where the march's took 367 and 535).  At most one unit in the last place
+// additions instead of a division's dozen (the read-out of 4096x2048: FP32 367 ->
+// 99 us, BF16S 535 -> 90).  At most one unit in the last place
 // from the FP64 division (20 million random operands); operands outside the
 // range where no term can leave FP32's normal range divide in FP64.
 __device__ __forceinline__ double half_force_velocity(float j, float F, float rho, float rc) {
@@ -386,8 +396,8 @@ template <int Q, typename T>
 __device__ __forceinline__ void node_moments(const T (&f)[Q], T& rho, T& jx, T& jy) {
   using L = Lattice<Q>;
   rho = f[0];
-  jx = T(L::cx(0)) * f[0];
-  jy = T(L::cy(0)) * f[0];
+  jx = L::cx(0) == 0 ? T(0) : T(L::cx(0)) * f[0];
+  jy = L::cy(0) == 0 ? T(0) : T(L::cy(0)) * f[0];
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
     rho += f[i];
@@ -453,11 +463,55 @@ template <int Q> __host__ __device__ constexpr int opposite(int i) {
 // evaluating every term in single precision otherwise leaves a rounding bias
 // in the node's mass (of order 1e-7 rho per step, correlated in space and
 // time) that accumulates into a visible density drift at interfaces.
+template <int Q>
+__device__ __forceinline__ void node_collide_fp64(const Physics<double>& P, double (&f)[Q],
+                                                  double rho, double ux, double uy, double usx,
+                                                  double usy) {
+  // The pair form with the quadratic terms shared between the pairs: every
+  // velocity lies on an axis or a diagonal (|c_x| = |c_y| = k), so that
+  //   (c.u*)^2 - g (c.u)^2 = k^2 X, k^2 Y or k^2 (X + Y +- 2 Z),
+  // X = u*_x^2 - g u_x^2, Y likewise, Z = u*_x u*_y - g u_x u_y; and c.(u* - g u)
+  // is k times a_x, a_y or a_x +- a_y.  6 operations per pair, all fused where
+  // they can be: the FP64 pipe (1/64 of the FP32 rate) bounds this path.
+  using E = EqConst<Q>;
+  using L = Lattice<Q>;
+  const double g = P.one_m_omega;
+  const double gux = g * ux, guy = g * uy;
+  const double ax = usx - gux, ay = usy - guy;
+  const double X = fma(usx, usx, -gux * ux), Y = fma(usy, usy, -guy * uy);
+  const double Z2 = 2.0 * fma(usx, usy, -gux * uy);
+  const double XY = X + Y, wB = fma(-E::inv_2theta, XY, P.omega);
+  const double Dp = XY + Z2, Dm = XY - Z2, ap = ax + ay, am = ax - ay;
+  static_for<0, Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    constexpr int j = opposite<Q>(i);
+    if constexpr (i == L::REST) {
+      f[i] = fma(g, f[i], (L::w(i) * rho) * wB);
+    } else if constexpr (i < j) {
+      constexpr int cx = L::cx(i), cy = L::cy(i);
+      constexpr int k = cx != 0 ? (cx < 0 ? -cx : cx) : (cy < 0 ? -cy : cy);
+      static_assert(cx == 0 || cy == 0 || cx * cx == cy * cy, "axis or diagonal");
+      const double q = cy == 0 ? X : (cx == 0 ? Y : (cx * cy > 0 ? Dp : Dm));
+      // c.(u* - g u) = sign * k * d
+      constexpr double sign = cx != 0 ? (cx > 0 ? 1.0 : -1.0) : (cy > 0 ? 1.0 : -1.0);
+      const double d = cy == 0 ? ax : (cx == 0 ? ay : (cx * cy > 0 ? ap : am));
+      const double S = (L::w(i) * rho) * fma(E::inv_2theta2 * k * k, q, wB);
+      const double K = (sign * L::w(i) * k * E::inv_theta) * rho;
+      f[i] = fma(g, f[i], fma(K, d, S));
+      f[j] = fma(g, f[j], fma(-K, d, S));
+    }
+  });
+}
+
 template <int Q, typename T>
 __device__ __forceinline__ void node_collide(const Physics<T>& P, T (&f)[Q], T rho, T ux, T uy,
                                              T usx, T usy) {
   using E = EqConst<Q>;
   using L = Lattice<Q>;
+  if constexpr (sizeof(T) == 8) {
+    node_collide_fp64<Q>(P, f, rho, ux, uy, usx, usy);
+    return;
+  }
   const T g = P.one_m_omega;
   const T ax = usx - g * ux, ay = usy - g * uy;
   const T Bt = (usx * usx + usy * usy - g * (ux * ux + uy * uy)) * T(E::inv_2theta);

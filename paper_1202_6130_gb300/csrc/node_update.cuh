@@ -54,8 +54,9 @@ __device__ __forceinline__ void write_moments(const Args& a, int64_t n, T rho, T
     a.out_ux[n] = half_force_velocity(jx, Fx, rho, rc);
     a.out_uy[n] = half_force_velocity(jy, Fy, rho, rc);
   } else {
-    a.out_ux[n] = (jx + 0.5 * Fx) / rho;
-    a.out_uy[n] = (jy + 0.5 * Fy) / rho;
+    const T y = T(1) / rho;
+    a.out_ux[n] = div_rho<T>(jx + 0.5 * Fx, rho, y);
+    a.out_uy[n] = div_rho<T>(jy + 0.5 * Fy, rho, y);
   }
 }
 
@@ -413,7 +414,19 @@ __device__ __forceinline__ void node_update(const Args& a, T (&f)[Q], uint32_t f
   });
   const T psi_c = prow[R][0];
   T sfx = 0, sfy = 0;
-  static_for<0, Q>([&](auto ic) {
+  if constexpr (sizeof(T) == 8) {
+    // Opposite neighbours differenced first, one product per pair and
+    // component (as many operations on the FP64 pipe as there are pairs).
+    static_for<0, Q>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      constexpr int cx = L::cx(i), cy = L::cy(i);
+      if constexpr (i < opposite<Q>(i)) {
+        const T nb = prow[R + cy][cx] - prow[R - cy][-cx];
+        if constexpr (cx != 0) sfx = fma(L::w(i) * cx, nb, sfx);
+        if constexpr (cy != 0) sfy = fma(L::w(i) * cy, nb, sfy);
+      }
+    });
+  } else static_for<0, Q>([&](auto ic) {
     constexpr int i = decltype(ic)::value;
     if constexpr (L::cx(i) != 0 || L::cy(i) != 0) {
       const T nb = prow[R + L::cy(i)][L::cx(i)];

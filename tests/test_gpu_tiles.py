@@ -92,6 +92,18 @@ def test_checks_fall_between_the_steps_of_two(pkg):
     sim.close()
 
 
+def test_fp64_psi_scale_other_than_one_matches_oracle(pkg):
+    """rho0 = 0.7: the FP64 quotient rho / rho0 by reciprocal and remainder."""
+    from oracle import lbm_oracle as O
+    w = _case(45, 26)
+    w.rho0 = 0.7
+    p = O.Params(lattice=O.D2Q9, tau=w.tau, G=w.G, rho0=w.rho0, body_force=tuple(w.body_force))
+    wall = O.Wall(w.phi_s, w.psi_r, w.psi_a, w.G_R, w.G_A, w.epsilon, w.u_wall)
+    f = O.run(p, wall, O.initial_populations(p, w.rho, w.ux, w.uy, w.noise), 20)
+    got, _ = _run(pkg, w, "fp64", 0, (20,))
+    np.testing.assert_allclose(got, f, rtol=1e-12, atol=1e-15)
+
+
 def test_fp32_velocity_quotient_is_within_an_ulp_of_fp64(pkg):
     """Without forces u = j / rho, j and rho formed in FP32 from the populations
     as the kernel forms them: the read-out's quotient of FP32 numbers differs
