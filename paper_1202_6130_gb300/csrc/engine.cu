@@ -32,11 +32,12 @@ struct lbm_ctx {
   int cur = 0;  // buffer holding the current state
   PopMaps tmap[2];       // population maps of buffer 0 and 1 (one per box depth): row march
   // Tile shapes (launch.cuh: tile_list) of one step (-1: the row march), of two
-  // steps per launch (-1: none) and of the read-out, with their maps per buffer.
-  enum { kOne, kTwo, kRead, kTiles };
-  int shape[kTiles] = {-1, -1, -1};
+  // steps per launch (-1: none), of the read-out and of the batch it was last a
+  // member of, with their maps per buffer.
+  enum { kOne, kTwo, kRead, kBatch, kTiles };
+  int shape[kTiles] = {-1, -1, -1, -1};
   PopMaps tile_map[kTiles][2];  // encoded on first use
-  bool tile_ready[kTiles] = {false, false, false};
+  bool tile_ready[kTiles] = {};
   // wall (compute precision: double for FP64 storage, float otherwise)
   void* wall_phie = nullptr;
   void* wall_sx = nullptr;
@@ -201,7 +202,7 @@ template <int Q, typename S> int make_tmap(lbm_ctx* c, int which) {
   return LBM_OK;
 }
 
-// Maps of tile use `use` (kOne, kTwo, kRead) for both population buffers.
+// Maps of tile use `use` for both population buffers.
 template <int Q, typename S> int ready_tile_maps(lbm_ctx* c, int use) {
   if (c->shape[use] < 0 || c->tile_ready[use]) return LBM_OK;
   EncodeFn enc = get_encode();
@@ -942,8 +943,9 @@ struct lbm_batch {
   std::vector<uint64_t> versions;
   std::vector<int> cur0;  // member cur at build time
   int Q = 0, storage = -1;
-  int tile_rows = 0;  // 0: each member's own choice
-  int ctas = 0;       // 0: one CTA per tile; > 0: that many persistent CTAs
+  int tile_rows = 0;  // 0: the engine's choice; > 0: row march, rows per segment
+  int ctas = 0;       // 0: one CTA per tile; > 0: row march by that many persistent CTAs
+  int shape = -1;     // tile shape of the members' kernel (-1: the row march)
   bool dirty = true;
   void* d_members = nullptr;
   size_t cap_members = 0;
@@ -1046,6 +1048,38 @@ void release_chunk(lbm_batch::Chunk& ch) {
   ch.done = nullptr;
 }
 
+// The default tiling of a batch: the one-step tile shape with the least estimated
+// time for all members (*rows = 0), or -1 and the rows per segment of a row march.
+// D2Q9 FP32 and 16-bit batches of more than about 12 rounds of 64x8 tiles march:
+// there a march's longer segments pay for their fill, and its arguments are read
+// once per segment instead of once per tile.  GB300, us per step, tiles / march of
+// the rows chosen: uneven FP16S lattices of 4.0 M nodes 50 / 57, 7.4 M 80 / 76,
+// 10.8 M 115 / 106, 22.0 M 234 / 203; FP32 65 / 71, 105 / 100, 150 / 140, 309 / 282.
+template <int Q, typename S> int batch_shape(const lbm_batch* b, int* rows) {
+  constexpr TileList list = tile_list<Q, S>();
+  double best = 1e30, rounds = 0.0;
+  int shape = -1;
+  for (int k = 0; k < list.n; ++k) {
+    const TileCfg& t = list.t[k];
+    if (t.steps != 1) continue;
+    int64_t tiles = 0;
+    for (const lbm_ctx* c : b->members)
+      tiles += (int64_t)((c->p.nx + t.tw - 1) / t.tw) * ((c->p.ny + t.th - 1) / t.th);
+    const double us = tile_cost<Q, S>(k, tiles);
+    if (us < best && tiles < (int64_t)1 << 30) {
+      best = us;
+      shape = k;
+      rounds = (double)tiles / tile_info<Q, S>(k).slots;
+    }
+  }
+  *rows = 0;
+  if (Q == 9 && sizeof(S) <= 4 && rounds > 12.0) {
+    *rows = std::clamp(4 * (int)std::lround(rounds / 8.0), 8, sizeof(S) == 4 ? 16 : 24);
+    return -1;
+  }
+  return shape;
+}
+
 template <int Q, typename S> int batch_build(lbm_batch* b) {
   using T = typename Codec<S>::T;
   using M = BatchMember<T, S>;
@@ -1055,14 +1089,24 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
   constexpr int kChunk = A::kChunk;
   const int nchunk = (n + kChunk - 1) / kChunk;
   std::vector<M> hm(n);
+  int rows = b->tile_rows;
+  b->shape = b->tile_rows == 0 && b->ctas == 0 ? batch_shape<Q, S>(b, &rows) : -1;
   b->versions.assign(n, 0);
   b->cur0.assign(n, 0);
   for (int i = 0; i < n; ++i) {
     lbm_ctx* c = b->members[i];
     M& m = hm[i];
     std::memset(&m, 0, sizeof m);
-    m.map[0] = c->tmap[0];
-    m.map[1] = c->tmap[1];
+    if (b->shape >= 0) {
+      if (c->shape[lbm_ctx::kBatch] != b->shape) {
+        c->shape[lbm_ctx::kBatch] = b->shape;
+        c->tile_ready[lbm_ctx::kBatch] = false;
+      }
+      if (ready_tile_maps<Q, S>(c, lbm_ctx::kBatch)) return bfail(b, LBM_ECUDA, "%s", c->err.c_str());
+    }
+    for (int d = 0; d < 2; ++d) m.map[d] = b->shape >= 0 ? c->tile_map[lbm_ctx::kBatch][d] : c->tmap[d];
+    m.flag_words = c->wall_flags;
+    m.flag_pitch = c->nchunk_pad;
     m.flags = c->has_wall ? c->flag_map : c->tmap[0].m[0];
     b->versions[i] = c->version;
     b->cur0[i] = c->cur;
@@ -1089,10 +1133,18 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
       for (int d = 0; d < 2; ++d)
         pa->a[i][d] = make_args<Q, S>(c, d, static_cast<S*>(c->buf[d ^ 1]), nullptr, nullptr, nullptr, 0);
       pa->cur[i] = c->cur;
+      if (b->shape >= 0) {
+        const TileCfg t = tile_list<Q, S>().t[b->shape];
+        pa->nseg[i] = (c->p.ny + t.th - 1) / t.th;
+        pa->nstrip[i] = (c->p.nx + t.tw - 1) / t.tw;
+        pa->tile0[i] = t0;
+        t0 += pa->nseg[i] * pa->nstrip[i];
+        continue;
+      }
       // Segments of about L rows, balanced over the member's height: a short
       // remainder segment would pay its 2R halo rows and its pipeline fill
       // for a few rows only.
-      const int L = std::max(1, std::min(b->tile_rows > 0 ? b->tile_rows : c->tile_rows, c->p.ny));
+      const int L = std::max(1, std::min(rows > 0 ? rows : c->tile_rows, c->p.ny));
       pa->nseg[i] = std::max(1, (c->p.ny + L / 2) / L);
       pa->nstrip[i] = (c->p.nx + W - 1) / W;
       pa->tile0[i] = t0;
@@ -1120,7 +1172,9 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
   }
   if (nchunk > 1 && !b->fork_ev) BCK(b, cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming));
   b->ntiles = (int)total;
-  batch_ctas_per_sm<Q, S>();  // sets the kernel's shared-memory attribute outside any capture
+  // The kernels' shared-memory attributes, outside any capture.
+  if (b->shape >= 0) BCK(b, prepare_batch_tiles<Q, S>(b->shape));
+  else batch_ctas_per_sm<Q, S>();
   int rc = bgrow(b, &b->d_members, &b->cap_members, sizeof(M) * std::max(1, n));
   if (rc) return rc;
   BCK(b, cudaMemcpyAsync(b->d_members, hm.data(), sizeof(M) * n, cudaMemcpyHostToDevice, b->stream));
@@ -1137,10 +1191,13 @@ template <int Q, typename S> cudaError_t batch_launch(lbm_batch* b, int parity) 
   using T = typename Codec<S>::T;
   const bool multi = b->chunks.size() > 1;
   for (const lbm_batch::Chunk& ch : b->chunks) {
-    cudaError_t e = launch_batch<Q, S>(
-        *reinterpret_cast<const BatchArgs<T, S>*>(ch.args.data()),
-        static_cast<const BatchMember<T, S>*>(b->d_members) + ch.base, ch.nctas, parity,
-        b->ctas > 0, ch.plain, multi ? ch.stream : b->stream);
+    const auto& args = *reinterpret_cast<const BatchArgs<T, S>*>(ch.args.data());
+    const auto* members = static_cast<const BatchMember<T, S>*>(b->d_members) + ch.base;
+    const cudaStream_t st = multi ? ch.stream : b->stream;
+    const cudaError_t e =
+        b->shape >= 0
+            ? launch_batch_tiles<Q, S>(b->shape, args, members, ch.nctas, parity, ch.plain, st)
+            : launch_batch<Q, S>(args, members, ch.nctas, parity, b->ctas > 0, ch.plain, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1404,7 +1461,8 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
   BCK(b, cudaGetDevice(&dev));
   BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int cps = dispatch(b->Q, b->storage, [&]<int Q, typename S>() { return batch_ctas_per_sm<Q, S>(); });
-  const int rows_c[] = {4, 8, 12, 16, 24, 32, 64};
+  // Row-march candidates, and (0, 0): the tiles that batch_build picks.
+  const int rows_c[] = {0, 4, 8, 12, 16, 24, 32, 64};
   const int ctas_c[] = {0, std::max(1, cps) * sms};
   cudaEvent_t e0, e1;
   BCK(b, cudaEventCreate(&e0));
@@ -1413,6 +1471,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
   int bt = b->tile_rows, bc = b->ctas;
   for (int tr : rows_c) {
     for (int ct : ctas_c) {
+      if (tr == 0 && ct != 0) continue;
       b->tile_rows = tr;
       b->ctas = ct;
       b->dirty = true;
@@ -1445,7 +1504,15 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tuned[tune_key(b)] = {bt, bc};
   }
-  if (best_tile_rows) *best_tile_rows = bt;
+  if (best_tile_rows) {
+    *best_tile_rows = bt;
+    if (bt == 0)  // rows per CTA of the default tiling
+      dispatch(b->Q, b->storage, [&]<int Q, typename S>() -> int {
+        const int shape = batch_shape<Q, S>(b, best_tile_rows);
+        if (shape >= 0) *best_tile_rows = tile_list<Q, S>().t[shape].th;
+        return LBM_OK;
+      });
+  }
   if (best_ctas) *best_ctas = bc;
   if (best_ms_per_step) *best_ms_per_step = best;
   return LBM_OK;

@@ -118,6 +118,14 @@ cudaError_t launch_batch(const BatchArgs<typename Codec<S>::T, S>& args,
                          int parity, bool persistent, bool plain, cudaStream_t stream);
 template <int Q, typename S> int batch_ctas_per_sm();
 
+// The same on tiles of shape `shape`, one CTA per tile.
+template <int Q, typename S>
+cudaError_t launch_batch_tiles(int shape, const BatchArgs<typename Codec<S>::T, S>& args,
+                               const BatchMember<typename Codec<S>::T, S>* members, int ntiles,
+                               int parity, bool plain, cudaStream_t stream);
+// Sets the shared-memory attribute of its kernels (outside any stream capture).
+template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape);
+
 // Auxiliary kernels (aux.cu).
 template <int Q, typename S>
 cudaError_t launch_encode(const double* f, S* buf, int nx, int ny, int64_t pitch, int64_t plane,

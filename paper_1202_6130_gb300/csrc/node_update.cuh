@@ -60,12 +60,19 @@ __device__ __forceinline__ void write_moments(const Args& a, int64_t n, T rho, T
   }
 }
 
-// Where a pair sits: its wall-field indices (used on flagged pairs), which of
-// its nodes count, and the coordinates that seed its rounding.
+// The rows of psi around a node: operator()(c_y) is the shared-memory row c_y above
+// it, at its column.  (A march passes the pointers themselves: computing them
+// on demand cost the batch march 4 registers and 7% of its time.)
+template <typename T, int R> struct PsiRows {
+  const T* row[2 * R + 1];
+  __device__ __forceinline__ const T* operator()(int cy) const { return row[R + cy]; }
+};
+
+// Where a pair sits in the lattice (its first node; for an image of a pair, the
+// pair itself), and which of its nodes exist.
 struct PairAt {
-  int64_t n0, n1;
+  int x, y;
   bool ok0, ok1;
-  uint32_t hx, hy;
 };
 
 // A pair's moments, velocity and total force.  f_: its stored values (f, or
@@ -162,7 +169,7 @@ template <int Q, typename S, bool EDGE = true> struct PairState {
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         if (e == 0 ? at.ok0 : at.ok1) {
-          const int64_t n = e == 0 ? at.n0 : at.n1;
+          const int64_t n = (int64_t)at.y * a.nx + at.x + e;
           phe[e] = a.wall.phie[n];
           Sx[e] = a.wall.sx[n];
           Sy[e] = a.wall.sy[n];
@@ -181,8 +188,6 @@ template <int Q, typename S, bool EDGE = true> struct PairState {
       Fx = fma2(mg, sfx, F2::splat(a.phys.bfx));
       Fy = fma2(mg, sfy, F2::splat(a.phys.bfy));
     }
-    if ((at.ok0 && !(fabsf(rho.x()) <= 3.0e38f)) || (at.ok1 && !(fabsf(rho.y()) <= 3.0e38f)))
-      atomicOr(a.status, kStatusNonFinite);
   }
 };
 
@@ -197,6 +202,8 @@ __device__ __forceinline__ void pair_collide(const Args& a, const St& n, F2 (&f_
   using PR = Pair<S>;
   using T = float;
   const F2 rho = n.rho, inv_rho = n.inv_rho, ux = n.ux, uy = n.uy;
+  if (!(fabsf(rho.x()) <= 3.0e38f) || (at.ok1 && !(fabsf(rho.y()) <= 3.0e38f)))
+    atomicOr(a.status, kStatusNonFinite);
   const F2 usx = fma2(n.Fx, inv_rho, ux);
   const F2 usy = fma2(n.Fy, inv_rho, uy);
   // EDM-BGK in pair form (see node_collide), packed over the two nodes
@@ -278,7 +285,7 @@ __device__ __forceinline__ void pair_collide(const Args& a, const St& n, F2 (&f_
   // the step).
   if constexpr (C::kShifted) {
     if (FL == kFlExpPlain || a.stochastic) {
-      const uint32_t h = sr_hash(at.hx, at.hy, key);
+      const uint32_t h = sr_hash((uint32_t)at.x, (uint32_t)at.y, key);
       static_for<0, Q>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         raw[i] = PR::store_sr(f_[i], h * sr_multiplier(i));
@@ -364,13 +371,7 @@ template <int Q, typename S, int MODE, int FL, bool EDGE = true, typename Args, 
 __device__ __forceinline__ void pair_update(const Args& a, F2 (&f_)[Q], const F2 Hm, uint32_t flag,
                                             int xp, int yo, bool strip_edge, bool simple_images,
                                             uint32_t key, Row&& psi_row) {
-  PairAt at;
-  at.n0 = (int64_t)yo * a.nx + xp;
-  at.n1 = at.n0 + 1;
-  at.ok0 = !EDGE || xp < a.nx;
-  at.ok1 = !EDGE || xp + 1 < a.nx;
-  at.hx = (uint32_t)xp;
-  at.hy = (uint32_t)yo;
+  const PairAt at{xp, yo, !EDGE || xp < a.nx, !EDGE || xp + 1 < a.nx};
   const PairState<Q, S, EDGE> n(a, f_, Hm, flag, at, psi_row);
   if (!at.ok0) return;
   if constexpr (MODE == kModeStep) {
@@ -378,10 +379,12 @@ __device__ __forceinline__ void pair_update(const Args& a, F2 (&f_)[Q], const F2
     pair_collide<Q, S, FL>(a, n, f_, Hm, at, key, raw);
     pair_store<Q, S, EDGE>(a, raw, xp, yo, strip_edge, simple_images);
   } else {
+    if (!(fabsf(n.rho.x()) <= 3.0e38f) || (at.ok1 && !(fabsf(n.rho.y()) <= 3.0e38f)))
+      atomicOr(a.status, kStatusNonFinite);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       if (e == 1 && !at.ok1) break;
-      const int64_t i = e == 0 ? at.n0 : at.n1;
+      const int64_t i = (int64_t)yo * a.nx + xp + e;
       const float r = e == 0 ? n.rho.x() : n.rho.y();
       write_moments(a, i, r, e == 0 ? n.jx.x() : n.jx.y(), e == 0 ? n.jy.x() : n.jy.y(),
                     e == 0 ? n.Fx.x() : n.Fx.y(), e == 0 ? n.Fy.x() : n.Fy.y());

@@ -200,6 +200,50 @@ template <int Q, typename S> int batch_ctas_per_sm() {
   return n;
 }
 
+template <int Q, typename S, int K, int FL> static cudaError_t prepare_batch_tile_k() {
+  using Cfg = TileConfig<Q, S, K>;
+  static cudaError_t once = cudaFuncSetAttribute(batch_tile_kernel<typename Cfg::Sh, FL, Cfg::kCfg.minb>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 Cfg::Sh::SMEM);
+  return once;
+}
+
+template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape) {
+  return with_shape<Q, S>(shape, [&]<int K>() {
+    if constexpr (TileConfig<Q, S, K>::kCfg.steps != 1) return cudaErrorInvalidValue;
+    else {
+    const cudaError_t e = prepare_batch_tile_k<Q, S, K, kFlExpPlain>();
+    return e != cudaSuccess ? e : prepare_batch_tile_k<Q, S, K, kFlRuntime>();
+    }
+  });
+}
+
+template <int Q, typename S>
+cudaError_t launch_batch_tiles(int shape, const BatchArgs<typename Codec<S>::T, S>& args,
+                               const BatchMember<typename Codec<S>::T, S>* members, int ntiles,
+                               int parity, bool plain, cudaStream_t stream) {
+  return with_shape<Q, S>(shape, [&]<int K>() {
+    using Cfg = TileConfig<Q, S, K>;
+    using Sh = typename Cfg::Sh;
+    if constexpr (Sh::TS != 1) {
+      return cudaErrorInvalidValue;
+    } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ntiles);
+    cfg.blockDim = dim3(Sh::NT);
+    cfg.dynamicSmemBytes = Sh::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return plain ? cudaLaunchKernelEx(&cfg, batch_tile_kernel<Sh, kFlExpPlain, Cfg::kCfg.minb>, args, members, parity)
+                 : cudaLaunchKernelEx(&cfg, batch_tile_kernel<Sh, kFlRuntime, Cfg::kCfg.minb>, args, members, parity);
+    }
+  });
+}
+
 }  // namespace lbm
 
 #define LBM_INSTANTIATE_STEP(Q, S)                                                         \
@@ -212,4 +256,8 @@ template <int Q, typename S> int batch_ctas_per_sm() {
   template cudaError_t lbm::launch_batch<Q, S>(                                          \
       const lbm::BatchArgs<lbm::Codec<S>::T, S>&,                                         \
       const lbm::BatchMember<lbm::Codec<S>::T, S>*, int, int, bool, bool, cudaStream_t);    \
+  template cudaError_t lbm::launch_batch_tiles<Q, S>(                                    \
+      int, const lbm::BatchArgs<lbm::Codec<S>::T, S>&,                                     \
+      const lbm::BatchMember<lbm::Codec<S>::T, S>*, int, int, bool, cudaStream_t);         \
+  template cudaError_t lbm::prepare_batch_tiles<Q, S>(int);                              \
   template int lbm::batch_ctas_per_sm<Q, S>();

@@ -558,11 +558,13 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
       }
 #pragma unroll
       for (int p = 0; p < P; ++p) {
-        pair_update<Q, S, kModeStep, FL>(
-            a, f[p], rho_cur[p], flag, x + 2 * p, yo, strip_edge, simple_images, key,
-            [&](int cy) -> const T* {  // ring row of node row yo + c_y
-              return ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + RO + xa + 2 * p;
-            });
+        PsiRows<T, R> rows;  // ring rows of node rows yo + c_y
+        static_for<0, 2 * R + 1>([&](auto rc) {
+          constexpr int cy = decltype(rc)::value - R;
+          rows.row[R + cy] = ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + RO + xa + 2 * p;
+        });
+        pair_update<Q, S, kModeStep, FL>(a, f[p], rho_cur[p], flag, x + 2 * p, yo, strip_edge,
+                                         simple_images, key, rows);
       }  // pairs
     }
     if (++s == NS) {
@@ -626,11 +628,14 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
                                (blockIdx.y & 1u) != 0u, sm, g, policy);
 }
 
-// A lattice of a batch: TMA maps of its two population buffers and of its wall
-// flags (in device memory; map[d] reads buffer d).
+// A lattice of a batch: TMA maps of its two population buffers for the batch's
+// kernel and of its wall flags, and the flag words themselves (in device memory;
+// map[d] reads buffer d).
 template <typename T, typename S> struct BatchMember {
   PopMaps map[2];
   CUtensorMap flags;
+  const uint32_t* flag_words;
+  int32_t flag_pitch;
 };
 
 // Step arguments of up to kChunk members of a batch for either direction
@@ -654,6 +659,15 @@ template <typename T, typename S> struct BatchArgs {
 static_assert(sizeof(BatchArgs<float, float>) <= 32764 && sizeof(BatchArgs<double, double>) <= 32764,
               "batch arguments fit the kernel parameter space");
 
+// The member that tile t of a chunk belongs to (uniform across the CTA: t comes
+// from the block index and the table from constant memory).
+template <typename Batch> __device__ __forceinline__ int batch_member(const Batch& P, int t) {
+  int m = 0;
+#pragma unroll
+  for (int j = 1; j < P.kChunk; ++j) m += t >= P.tile0[j] ? 1 : 0;
+  return m;
+}
+
 // One time step of up to kChunk lattices of a batch.  Tile t is segment
 // t / nstrip (rows balanced over the member's height, odd segments marched
 // upwards as in step_kernel) and strip t % nstrip of its member.  With
@@ -674,9 +688,7 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
   griddep_launch_dependents();
   griddep_wait();
   auto march_tile = [&](int t) -> bool {
-    int m = 0;
-#pragma unroll
-    for (int j = 1; j < P.kChunk; ++j) m += t >= P.tile0[j] ? 1 : 0;
+    const int m = batch_member(P, t);
     const int local = t - P.tile0[m];
     const int seg = local / P.nstrip[m];
     const int x0 = (local - seg * P.nstrip[m]) * W;

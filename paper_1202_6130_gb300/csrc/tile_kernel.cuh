@@ -32,6 +32,7 @@
 #pragma once
 
 #include "node_update.cuh"
+#include "step_kernel.cuh"
 #include "tma.cuh"
 
 namespace lbm {
@@ -284,13 +285,7 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
                                       key + (uint32_t)s, psi_row);
         } else {
           // Even nx: the pair and its periodic images are pairs of whole nodes.
-          const int xw = E ? wrap_x(x) : x, yw = E ? wrap_y(y) : y;
-          PairAt at;
-          at.n0 = (int64_t)yw * a.nx + xw;
-          at.n1 = at.n0 + 1;
-          at.ok0 = at.ok1 = true;
-          at.hx = (uint32_t)xw;
-          at.hy = (uint32_t)yw;
+          const PairAt at{E ? wrap_x(x) : x, E ? wrap_y(y) : y, true, true};
           const PairState<Q, S, E> n(a, f[k], H[k], flag[k], at, psi_row);
           typename Pair<S>::Raw raw[Q];
           pair_collide<Q, S, FL>(a, n, f[k], H[k], at, key + (uint32_t)s, raw);
@@ -332,6 +327,25 @@ __global__ void __launch_bounds__(Sh::NT, MINB)
                             smem_raw);
   if constexpr (MODE == kModeStep)
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<MODE>(a, Sh::TS);
+}
+
+// One step of up to kChunk lattices of a batch on tiles: CTA b updates tile b of
+// the chunk, numbered member by member and, within a member, row by row
+// (nstrip tiles per row).  Members and arguments as for batch_step_kernel.
+template <typename Sh, int FL, int MINB>
+__global__ void __launch_bounds__(Sh::NT, MINB)
+    batch_tile_kernel(const __grid_constant__ BatchArgs<typename Sh::T, typename Sh::S> P,
+                      const BatchMember<typename Sh::T, typename Sh::S>* __restrict__ members,
+                      int32_t parity) {
+  extern __shared__ unsigned char smem_raw[];
+  const int m = batch_member(P, (int)blockIdx.x);
+  const int local = (int)blockIdx.x - P.tile0[m], ty = local / P.nstrip[m];
+  const int dir = (P.cur[m] ^ parity) & 1;
+  const auto& a = P.a[m][dir];
+  const auto* mb = &members[m];
+  tile_update<Sh, kModeStep, FL>(&mb->map[dir], mb->flag_words, mb->flag_pitch, a,
+                                 (local - ty * P.nstrip[m]) * Sh::TW, ty * Sh::TH, smem_raw);
+  if (threadIdx.x == 0 && local == 0) advance_key<kModeStep>(a, Sh::TS);
 }
 
 }  // namespace lbm
