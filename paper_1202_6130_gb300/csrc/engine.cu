@@ -226,34 +226,40 @@ template <int Q, typename S> int ready_tile_maps(lbm_ctx* c, int use) {
   return LBM_OK;
 }
 
-// Estimated microseconds per launch of tile shape k on the given lattices: the
-// rounds of resident CTAs it takes, the last one counted whole while there are
-// few, plus the launch and the first loads.
+// Estimated microseconds of a launch of `tiles` tiles of shape k.  FP64 is bound by
+// the FP64 pipe of the SM with the most tiles; the others by latency, which
+// further CTAs on an SM share.
 template <int Q, typename S> double tile_cost(int k, int64_t tiles) {
   const TileInfo t = tile_info<Q, S>(k);
   if (t.slots <= 0) return 1e30;
-  const double r = (double)tiles / t.slots;
-  return 1.2 + tile_list<Q, S>().t[k].us * (r < 4.0 ? std::ceil(r) : r + 0.5);
+  constexpr TileList list = tile_list<Q, S>();
+  const TileCfg& c = list.t[k];
+  if (sizeof(S) == 8) return c.us0 + c.us * (double)((tiles + t.sms - 1) / t.sms);
+  return c.us0 + c.us * (double)std::max<int64_t>(tiles, t.sms) / t.slots;
 }
 
-// Picks the tile shapes of a lattice, all by estimated time per step.  One row
-// march stays ahead of the one-step tiles: D2Q9 FP32 on lattices whose two
-// buffers exceed L2 twice over, which HBM bounds (8192x4096: 0.368 ms against
-// 0.399; 4096x2048: 0.0963 against 0.0983).  Two steps per launch need whole node pairs under
-// periodic wrapping (even nx) and a lattice no smaller than the halo; an
-// explicit tile_rows asks for the row march.
+// Picks the tile shapes of a lattice by estimated time per step.  One row march
+// stays ahead of the one-step tiles: D2Q9 FP32 and 16-bit lattices whose
+// populations exceed L2 (FP32 twice over, 16-bit four times), which HBM or the
+// issue slots bound and not latency (GB300, us per step, march / tiles: FP32
+// 8192x4096 367 / 400, 4096x2048 97 / 101; FP16S 234 / 237, BF16S 234 / 243, but
+// 4096x2048 FP16S 68 / 62).  Two steps per launch beat the march for FP32 (291),
+// not for 16-bit storage (261).  They need whole node pairs under periodic
+// wrapping (even nx) and a lattice no smaller than the halo; an explicit tile_rows
+// asks for the row march.
 template <int Q, typename S> void choose_tiles(lbm_ctx* c) {
   constexpr TileList list = tile_list<Q, S>();
   c->shape[lbm_ctx::kRead] = list.moments;
   if (c->p.tile_rows > 0) return;
   const int64_t nodes = (int64_t)c->p.nx * c->p.ny;
-  const bool march = Q == 9 && sizeof(S) == 4 && 2 * Q * (int64_t)sizeof(S) * nodes > (int64_t)260 << 20;
+  const bool march = Q == 9 && ((sizeof(S) == 4 && nodes > (int64_t)4 << 20) ||
+                                (sizeof(S) == 2 && nodes > (int64_t)16 << 20));
   double best[2] = {1e30, 1e30};
   for (int k = 0; k < list.n; ++k) {
     const TileCfg& t = list.t[k];
     const int use = t.steps == 2 ? lbm_ctx::kTwo : lbm_ctx::kOne;
     if (use == lbm_ctx::kTwo && (c->p.nx % 2 || c->p.nx < 4 || c->p.ny < 4)) continue;
-    if (use == lbm_ctx::kOne && march) continue;
+    if (march && (use == lbm_ctx::kOne || sizeof(S) == 2)) continue;
     const int64_t tiles = (int64_t)((c->p.nx + t.tw - 1) / t.tw) * ((c->p.ny + t.th - 1) / t.th);
     const double us = tile_cost<Q, S>(k, tiles) / t.steps;
     if (us < best[use]) {

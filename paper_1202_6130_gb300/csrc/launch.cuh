@@ -54,17 +54,18 @@ cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
 
 // Shapes of the tile kernel per (lattice, storage): tile width and height,
 // threads, time steps per launch, whether tiles without edges or walls run a
-// copy of the update without that code, CTAs per SM the registers are sized
-// for, and the microseconds one round of resident CTAs takes (GB300, lattices
-// of 2048x1024 and larger).  choose_tiles picks the shape with the least
-// estimated time, rounds x this figure, per time step.
+// copy of the update without that code, CTAs per SM the registers are sized for,
+// and the microseconds of a launch, us0 + us per round of resident CTAs (FP64: per
+// tile of the SM with the most tiles), fitted to GB300 times on 128x64 to 4096x2048 lattices (within about 15%).  The shape with
+// the least time per step by this estimate runs (choose_tiles); on the lattices
+// of the fit that is the fastest one or within 6% of it.
 struct TileCfg {
   int tw, th, nt, steps;
   bool in;
   int minb;
-  double us;
+  double us0, us;
 };
-constexpr int kMaxTileShapes = 6;
+constexpr int kMaxTileShapes = 7;
 struct TileList {
   TileCfg t[kMaxTileShapes];
   int n;
@@ -72,19 +73,36 @@ struct TileList {
 };
 template <int Q, typename S> constexpr TileList tile_list() {
   if constexpr (sizeof(S) == 8 && Q == 9)
-    return {{{16, 4, 64, 1, false, 4, 18.0}, {32, 8, 256, 1, false, 3, 29.7}, {32, 16, 256, 1, true, 2, 38.4}}, 3, 2};
+    return {{{16, 4, 64, 1, false, 4, 5.6, 2.8},
+             {32, 8, 256, 1, false, 3, 3.8, 9.85},
+             {32, 16, 256, 1, true, 2, 4.7, 19.1}}, 3, 2};
   else if constexpr (sizeof(S) == 8)
-    return {{{16, 4, 64, 1, false, 4, 48.0}, {32, 8, 256, 1, false, 3, 62.0}, {32, 16, 256, 1, true, 2, 80.0}}, 3, 2};
+    return {{{16, 4, 64, 1, false, 4, 10.0, 5.95},
+             {32, 8, 256, 1, false, 3, 5.3, 19.6},
+             {32, 16, 256, 1, true, 2, 2.0, 39.0}}, 3, 2};
   else if constexpr (Q == 21 && sizeof(S) == 4)
-    return {{{16, 4, 64, 1, false, 4, 3.0}, {32, 8, 256, 1, false, 3, 4.3}, {64, 8, 256, 1, true, 2, 5.2}}, 3, 1};
+    return {{{16, 4, 64, 1, false, 4, 3.9, 3.3},
+             {32, 8, 256, 1, false, 3, 3.2, 4.1},
+             {64, 8, 256, 1, true, 2, 6.0, 4.7}}, 3, 1};
   else if constexpr (Q == 21)
-    return {{{32, 4, 64, 1, false, 8, 4.1}, {64, 8, 128, 1, true, 4, 6.9}}, 2, 1};
+    return {{{32, 4, 64, 1, false, 8, 3.6, 3.85},
+             {64, 8, 128, 1, true, 4, 6.0, 5.6}}, 2, 1};
   else if constexpr (sizeof(S) == 4)
-    return {{{32, 4, 64, 1, false, 8, 2.8}, {64, 8, 128, 1, true, 7, 6.4}, {32, 4, 160, 2, false, 4, 3.05},
-             {32, 8, 224, 2, false, 3, 3.5}, {64, 12, 288, 2, true, 3, 6.8}, {64, 24, 320, 2, true, 2, 8.8}}, 6, 0};
+    return {{{32, 4, 64, 1, false, 8, 2.4, 2.6},
+             {64, 8, 128, 1, true, 7, 2.3, 6.6},
+             {32, 4, 160, 2, false, 4, 2.0, 3.35},
+             {32, 8, 224, 2, false, 3, 2.6, 3.9},
+             {32, 16, 192, 2, true, 4, 5.3, 6.0},
+             {64, 12, 288, 2, true, 3, 5.0, 6.8},
+             {64, 24, 320, 2, true, 2, 7.0, 8.3}}, 7, 0};
   else
-    return {{{32, 4, 64, 1, false, 8, 2.5}, {64, 8, 128, 1, true, 7, 4.1}, {32, 4, 160, 2, false, 4, 3.4},
-             {32, 8, 224, 2, false, 3, 3.2}, {64, 12, 288, 2, true, 3, 6.0}, {64, 24, 320, 2, true, 2, 7.6}}, 6, 0};
+    return {{{32, 4, 64, 1, false, 8, 2.2, 2.9},
+             {64, 8, 128, 1, true, 7, 3.4, 3.9},
+             {32, 4, 160, 2, false, 4, 1.7, 3.2},
+             {32, 8, 224, 2, false, 3, 2.5, 3.3},
+             {32, 16, 192, 2, true, 4, 4.7, 5.4},
+             {64, 12, 288, 2, true, 3, 4.6, 5.8},
+             {64, 24, 320, 2, true, 2, 6.7, 7.2}}, 7, 0};
 }
 template <int Q, typename S, int K> struct TileConfig {
   static constexpr TileCfg kCfg = tile_list<Q, S>().t[K];
@@ -100,7 +118,7 @@ cudaError_t launch_tile(int shape, const PopMaps& src, const uint32_t* flags, in
 // What the host needs of a tile shape: its TMA boxes, and the tiles that one
 // round of resident CTAs takes (0 if the kernel cannot run).
 struct TileInfo {
-  int bw, bh, nmap, depth[kMaxMaps], slots;
+  int bw, bh, nmap, depth[kMaxMaps], slots, sms;
 };
 template <int Q, typename S> TileInfo tile_info(int shape);
 

@@ -75,10 +75,48 @@ struct PairAt {
   bool ok0, ok1;
 };
 
+// The wall fields of a pair (phi_S^eps, S, U_wall; zero where a node does not
+// exist), and of a node.
+struct PairWall {
+  F2 phe, Sx, Sy, ux, uy;
+};
+template <typename Args> __device__ __forceinline__ PairWall load_wall(const Args& a, const PairAt& at) {
+  float v[5][2] = {};
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    if (e == 0 ? at.ok0 : at.ok1) {
+      const int64_t n = (int64_t)at.y * a.nx + at.x + e;
+      v[0][e] = a.wall.phie[n];
+      v[1][e] = a.wall.sx[n];
+      v[2][e] = a.wall.sy[n];
+      if (a.wall.uwx) {
+        v[3][e] = a.wall.uwx[n];
+        v[4][e] = a.wall.uwy[n];
+      }
+    }
+  }
+  return {F2(v[0][0], v[0][1]), F2(v[1][0], v[1][1]), F2(v[2][0], v[2][1]), F2(v[3][0], v[3][1]),
+          F2(v[4][0], v[4][1])};
+}
+template <typename T> struct NodeWall {
+  T phe, Sx, Sy, ux, uy;
+};
+template <typename T, typename Args>
+__device__ __forceinline__ NodeWall<T> load_wall(const Args& a, int x, int y) {
+  const int64_t n = (int64_t)y * a.nx + x;
+  NodeWall<T> w{a.wall.phie[n], a.wall.sx[n], a.wall.sy[n], T(0), T(0)};
+  if (a.wall.uwx) {
+    w.ux = a.wall.uwx[n];
+    w.uy = a.wall.uwy[n];
+  }
+  return w;
+}
+
 // A pair's moments, velocity and total force.  f_: its stored values (f, or
 // h = sigma (f - w rho_s) for 16-bit storage); Hm: their sum in table order.
 // psi_row(c_y): the shared-memory row of psi at c_y rows above, at the pair's
-// first column.  flag: non-zero where wall terms act.
+// first column.  flag: non-zero where wall terms act; wall(): the wall fields,
+// called there only.
 template <int Q, typename S, bool EDGE = true> struct PairState {
   using L = Lattice<Q>;
   using C = Codec<S>;
@@ -86,9 +124,9 @@ template <int Q, typename S, bool EDGE = true> struct PairState {
   static constexpr T kInvScale = PairRho<S>::kInvScale;
   F2 rho, inv_rho, ux, uy, Jx, Jy, jx, jy, Fx, Fy;
 
-  template <typename Args, typename Row>
+  template <typename Args, typename Row, typename Wall>
   __device__ __forceinline__ PairState(const Args& a, const F2 (&f_)[Q], const F2 Hm, uint32_t flag,
-                                       const PairAt& at, Row&& psi_row) {
+                                       Row&& psi_row, Wall&& wall) {
     // J = sum f_i c_i (D2Q9: the diagonal differences f5 - f7 and f8 - f6 shared
     // by its two components; otherwise in table order), j = J / sigma (the
     // shifts carry no momentum).
@@ -165,25 +203,12 @@ template <int Q, typename S, bool EDGE = true> struct PairState {
     const F2 mg = F2::splat(-a.phys.G) * psi_c;
     if (EDGE && flag != 0u) {
       const F2 ffx = mg * sfx, ffy = mg * sfy;
-      T phe[2] = {0, 0}, Sx[2] = {0, 0}, Sy[2] = {0, 0}, wx[2] = {0, 0}, wy[2] = {0, 0};
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        if (e == 0 ? at.ok0 : at.ok1) {
-          const int64_t n = (int64_t)at.y * a.nx + at.x + e;
-          phe[e] = a.wall.phie[n];
-          Sx[e] = a.wall.sx[n];
-          Sy[e] = a.wall.sy[n];
-          if (a.wall.uwx) {
-            wx[e] = a.wall.uwx[n];
-            wy[e] = a.wall.uwy[n];
-          }
-        }
-      }
-      const F2 rp = rho * F2(phe[0], phe[1]);
-      const F2 dfx = rp * (F2(wx[0], wx[1]) - ux - ffx * inv_rho);
-      const F2 dfy = rp * (F2(wy[0], wy[1]) - uy - ffy * inv_rho);
-      Fx = ((ffx + rho * F2(Sx[0], Sx[1])) + dfx) + F2::splat(a.phys.bfx);
-      Fy = ((ffy + rho * F2(Sy[0], Sy[1])) + dfy) + F2::splat(a.phys.bfy);
+      const PairWall w = wall();
+      const F2 rp = rho * w.phe;
+      const F2 dfx = rp * (w.ux - ux - ffx * inv_rho);
+      const F2 dfy = rp * (w.uy - uy - ffy * inv_rho);
+      Fx = ((ffx + rho * w.Sx) + dfx) + F2::splat(a.phys.bfx);
+      Fy = ((ffy + rho * w.Sy) + dfy) + F2::splat(a.phys.bfy);
     } else {
       Fx = fma2(mg, sfx, F2::splat(a.phys.bfx));
       Fy = fma2(mg, sfy, F2::splat(a.phys.bfy));
@@ -301,14 +326,16 @@ __device__ __forceinline__ void pair_collide(const Args& a, const St& n, F2 (&f_
 }
 
 // The primary store of a pair at (xp, yo) plus its periodic images.
+// LANES: on lattices of odd width whose nodes have at most one image column and
+// row, the images go out node by node without the general loop.
 // strip_edge: the pair may lie within GX of a side; simple_images: every pair
 // has at most one image column and one image row, and they are pairs again.
-template <int Q, typename S, bool EDGE = true, typename Args>
+template <int Q, typename S, bool LANES, typename Args>
 __device__ __forceinline__ void pair_store(const Args& a, const typename Pair<S>::Raw (&raw)[Q],
                                            int xp, int yo, bool strip_edge, bool simple_images) {
   using PR = Pair<S>;
   constexpr int GX = ghost_x<S, Lattice<Q>::R>(), GY = ghost_y<Lattice<Q>::R>();
-  const bool pair_ok = !EDGE || xp + 1 < a.nx;  // both nodes exist
+  const bool pair_ok = xp + 1 < a.nx;  // both nodes exist
   S* out = a.fout + (int64_t)(yo + GY) * a.pitch + xp + GX;
   if (pair_ok) {
     static_for<0, Q>([&](auto ic) {
@@ -322,7 +349,6 @@ __device__ __forceinline__ void pair_store(const Args& a, const typename Pair<S>
       out[Planes<Q>::template plane<i> * a.plane] = PR::lane(raw[i], 0);
     });
   }
-  if constexpr (!EDGE) return;
   const bool xedge = strip_edge && (xp < GX || xp + 1 >= a.nx - GX);
   const bool yedge = yo < GY || yo >= a.ny - GY;
   if ((xedge || yedge) && pair_ok && simple_images) {
@@ -341,6 +367,24 @@ __device__ __forceinline__ void pair_store(const Args& a, const typename Pair<S>
     if (sy != 0) {
       put(sy);
       if (sx != 0) put(sy + sx);
+    }
+  } else if (LANES && (xedge || yedge) && a.nx >= 2 * GX && a.ny >= 2 * GY) {
+    const int64_t sy = !yedge ? 0 : (int64_t)(yo < GY ? a.ny : -a.ny) * a.pitch;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (xp + e >= a.nx) break;
+      const int sx = xp + e < GX ? a.nx : (xp + e >= a.nx - GX ? -a.nx : 0);
+      auto put = [&](int64_t d) {
+        static_for<0, Q>([&](auto ic) {
+          constexpr int i = decltype(ic)::value;
+          out[d + e + Planes<Q>::template plane<i> * a.plane] = PR::lane(raw[i], e);
+        });
+      };
+      if (sx != 0) put(sx);
+      if (sy != 0) {
+        put(sy);
+        if (sx != 0) put(sy + sx);
+      }
     }
   } else if (xedge || yedge) {
 #pragma unroll 1
@@ -365,19 +409,32 @@ __device__ __forceinline__ void pair_store(const Args& a, const typename Pair<S>
   }
 }
 
+// The store of a pair without images, off elements after org: with the CTA's
+// origin and the pair's offset in it kept apart, a plane's address is a base that
+// the CTA shares plus one 32-bit offset.
+template <int Q, typename S, typename Args>
+__device__ __forceinline__ void pair_store_inside(const Args& a, const typename Pair<S>::Raw (&raw)[Q],
+                                                  S* org, uint32_t off) {
+  static_for<0, Q>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    char* base = reinterpret_cast<char*>(org + Planes<Q>::template plane<i> * a.plane);
+    *reinterpret_cast<typename Pair<S>::Raw*>(base + off * (uint32_t)sizeof(S)) = raw[i];
+  });
+}
+
 // Updates the node pair (xp, yo), (xp + 1, yo) and stores the result
 // (kModeStep) or the moments (kModeMoments).
-template <int Q, typename S, int MODE, int FL, bool EDGE = true, typename Args, typename Row>
+template <int Q, typename S, int MODE, int FL, bool LANES, typename Args, typename Row, typename Wall>
 __device__ __forceinline__ void pair_update(const Args& a, F2 (&f_)[Q], const F2 Hm, uint32_t flag,
                                             int xp, int yo, bool strip_edge, bool simple_images,
-                                            uint32_t key, Row&& psi_row) {
-  const PairAt at{xp, yo, !EDGE || xp < a.nx, !EDGE || xp + 1 < a.nx};
-  const PairState<Q, S, EDGE> n(a, f_, Hm, flag, at, psi_row);
+                                            uint32_t key, Row&& psi_row, Wall&& wall) {
+  const PairAt at{xp, yo, xp < a.nx, xp + 1 < a.nx};
+  const PairState<Q, S> n(a, f_, Hm, flag, psi_row, wall);
   if (!at.ok0) return;
   if constexpr (MODE == kModeStep) {
     typename Pair<S>::Raw raw[Q];
     pair_collide<Q, S, FL>(a, n, f_, Hm, at, key, raw);
-    pair_store<Q, S, EDGE>(a, raw, xp, yo, strip_edge, simple_images);
+    pair_store<Q, S, LANES>(a, raw, xp, yo, strip_edge, simple_images);
   } else {
     if (!(fabsf(n.rho.x()) <= 3.0e38f) || (at.ok1 && !(fabsf(n.rho.y()) <= 3.0e38f)))
       atomicOr(a.status, kStatusNonFinite);
@@ -395,9 +452,10 @@ __device__ __forceinline__ void pair_update(const Args& a, F2 (&f_)[Q], const F2
 // Updates the node (x, yo) from its populations f and stores the result
 // (kModeStep) or the moments (kModeMoments).  Arguments as for pair_update.
 template <int Q, typename S, int MODE, int FL, bool EDGE = true, typename T, typename Args,
-          typename Row>
+          typename Row, typename Wall>
 __device__ __forceinline__ void node_update(const Args& a, T (&f)[Q], uint32_t flag, int x, int yo,
-                                            bool strip_edge, bool simple_images, Row&& psi_row) {
+                                            bool strip_edge, bool simple_images, Row&& psi_row,
+                                            Wall&& wall) {
   using L = Lattice<Q>;
   using C = Codec<S>;
   constexpr int R = L::R;
@@ -441,19 +499,10 @@ __device__ __forceinline__ void node_update(const Args& a, T (&f)[Q], uint32_t f
 
   // Wall terms only on flagged (row, 32-column chunk) pairs.
   const bool has_wall = EDGE && flag != 0u && x < a.nx;
-  T phie = 0, Sx = 0, Sy = 0, uwx = 0, uwy = 0;
-  if (has_wall) {
-    const int64_t n = (int64_t)yo * a.nx + x;
-    phie = a.wall.phie[n];
-    Sx = a.wall.sx[n];
-    Sy = a.wall.sy[n];
-    if (a.wall.uwx) {
-      uwx = a.wall.uwx[n];
-      uwy = a.wall.uwy[n];
-    }
-  }
+  NodeWall<T> w{};
+  if (has_wall) w = wall();
   T Fx, Fy;
-  node_force<T>(a.phys, rho, ux, uy, psi_c, sfx, sfy, has_wall, phie, Sx, Sy, uwx, uwy,
+  node_force<T>(a.phys, rho, ux, uy, psi_c, sfx, sfy, has_wall, w.phe, w.Sx, w.Sy, w.ux, w.uy,
                 inv_rho, Fx, Fy);
 
   if (!EDGE || x < a.nx) {

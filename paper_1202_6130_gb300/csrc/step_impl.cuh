@@ -64,6 +64,31 @@ static cudaError_t prepare_tile() {
   return once;
 }
 
+static int sm_count() {
+  static int sms = [] {
+    int dev = 0, n = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
+               ? n : 0;
+  }();
+  return sms;
+}
+
+// CTAs of the K-th shape that the GPU holds at once (0 if the kernel cannot run).
+template <int Q, typename S, int K> static int tile_slots() {
+  using Cfg = TileConfig<Q, S, K>;
+  using Sh = typename Cfg::Sh;
+  static int slots = [] {
+    int n = 0;
+    if (prepare_tile<Q, S, K, kModeStep, kFlExpPlain>() != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &n, tile_kernel<Sh, kModeStep, kFlExpPlain, Cfg::kCfg.minb>, Sh::NT, Sh::SMEM) != cudaSuccess)
+      return 0;
+    return n * sm_count();
+  }();
+  return slots;
+}
+
 template <int Q, typename S, int K, int MODE, int FL>
 static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int flag_pitch,
                                  const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream) {
@@ -73,6 +98,8 @@ static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int 
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW, (a.ny + Sh::TH - 1) / Sh::TH);
+  const int slots = Sh::IN ? tile_slots<Q, S, K>() : 0;
+  const int ahead = (int64_t)cfg.gridDim.x * cfg.gridDim.y > slots ? slots / 2 : 0;
   cfg.blockDim = dim3(Sh::NT);
   cfg.dynamicSmemBytes = Sh::SMEM;
   cfg.stream = stream;
@@ -81,7 +108,7 @@ static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tile_kernel<Sh, MODE, FL, Cfg::kCfg.minb>, src, flags, flag_pitch, a);
+  return cudaLaunchKernelEx(&cfg, tile_kernel<Sh, MODE, FL, Cfg::kCfg.minb>, src, flags, flag_pitch, ahead, a);
 }
 
 // Calls fn<K>() for the K-th shape of the list.
@@ -107,19 +134,10 @@ template <int Q, typename S> TileInfo tile_info(int shape) {
   return with_shape<Q, S>(shape, [&]<int K>() {
     using Cfg = TileConfig<Q, S, K>;
     using Sh = typename Cfg::Sh;
-    TileInfo t{Sh::BW, Sh::BH, Sh::NMAP, {}, 0};
+    TileInfo t{Sh::BW, Sh::BH, Sh::NMAP, {}, 0, 0};
     for (int k = 0; k < Sh::NMAP; ++k) t.depth[k] = Sh::kTab.depth[k];
-    static int slots = [] {
-      int n = 0, dev = 0, sms = 0;
-      if (prepare_tile<Q, S, K, kModeStep, kFlExpPlain>() != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-              &n, tile_kernel<Sh, kModeStep, kFlExpPlain, Cfg::kCfg.minb>, Sh::NT, Sh::SMEM) != cudaSuccess ||
-          cudaGetDevice(&dev) != cudaSuccess ||
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 0;
-      return n * sms;
-    }();
-    t.slots = slots;
+    t.slots = tile_slots<Q, S, K>();
+    t.sms = sm_count();
     return t;
   });
 }

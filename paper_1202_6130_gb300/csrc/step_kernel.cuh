@@ -342,7 +342,8 @@ __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensor
           a, f, flag, x, yo, strip_edge, simple_images,
           [&](int cy) -> const T* {  // ring row of node row yo + c_y
             return ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + tid + Sh::RO;
-          });
+          },
+          [&] { return load_wall<T>(a, x, yo); });
     }
     if (++s == NS) {
       s = 0;
@@ -563,8 +564,9 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
           constexpr int cy = decltype(rc)::value - R;
           rows.row[R + cy] = ring + ((ko + ds * cy) & (Sh::RING_H - 1)) * Sh::RING_W + RO + xa + 2 * p;
         });
-        pair_update<Q, S, kModeStep, FL>(a, f[p], rho_cur[p], flag, x + 2 * p, yo, strip_edge,
-                                         simple_images, key, rows);
+        pair_update<Q, S, kModeStep, FL, false>(
+            a, f[p], rho_cur[p], flag, x + 2 * p, yo, strip_edge, simple_images, key, rows,
+            [&] { return load_wall(a, PairAt{x + 2 * p, yo, x + 2 * p < a.nx, x + 2 * p + 1 < a.nx}); });
       }  // pairs
     }
     if (++s == NS) {

@@ -119,11 +119,12 @@ template <int Q_, typename S_, int TW_, int TH_, int NT_, int TS_, bool IN_> str
 };
 
 // Advances the tile with origin (x0, y0) by TS time steps (kModeStep), or writes
-// its moments (kModeMoments, TS = 1).
+// its moments (kModeMoments, TS = 1).  (xn, yn): a later CTA's tile to fetch into
+// L2 meanwhile (xn < 0: none).
 template <typename Sh, int MODE, int FL, typename Args>
 __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* __restrict__ flags,
                                             int flag_pitch, const Args& a, int x0, int y0,
-                                            unsigned char* smem_raw) {
+                                            int xn, int yn, unsigned char* smem_raw) {
   using S = typename Sh::S;
   using T = typename Sh::T;
   using C = Codec<S>;
@@ -144,6 +145,55 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
     fence_barrier_init();
     static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src->m[decltype(kc)::value]); });
   }
+  auto wrap_x = [&](int x) { return x < 0 ? x + a.nx : (x >= a.nx ? x - a.nx : x); };
+  auto wrap_y = [&](int y) { return y < 0 ? y + a.ny : (y >= a.ny ? y - a.ny : y); };
+  // Column and row of the thread's k-th item of step s, whether it is updated
+  // (its nodes exist, or are images of nodes), and its wall flag.
+  auto item = [&](auto sc, int k, int& col, int& row) -> bool {
+    constexpr int s = decltype(sc)::value;
+    constexpr int M = Sh::margin(s), PROW = Sh::prow(s), NI = Sh::items(s);
+    if constexpr (NT % PROW == 0) {  // every slot in the thread's first column
+      row = tid / PROW + k * (NT / PROW) - M;
+      col = V * (tid % PROW) - M;
+    } else {
+      const int p = tid + k * NT, q = p / PROW;
+      row = q - M;
+      col = V * (p - q * PROW) - M;
+    }
+    return (NI % NT == 0 || tid + k * NT < NI) && x0 + col < a.nx + M && y0 + row < a.ny + M;
+  };
+  auto flag_of = [&](auto sc, bool on, int col, int row) -> uint32_t {
+    constexpr int M = Sh::margin(decltype(sc)::value);
+    if (!a.wall.active || !on) return 0u;
+    const int xw = M ? wrap_x(x0 + col) : x0 + col, yw = M ? wrap_y(y0 + row) : y0 + row;
+    return flags[(int64_t)yw * flag_pitch + (xw >> 5)];
+  };
+  // Shapes for small lattices (one item per thread and step, every tile at an
+  // edge or a wall) fetch the flags and wall fields of all steps ahead of the
+  // wait for the previous launch: set_wall ran to its end before this launch was
+  // enqueued, so they are static, and their latency leaves the step's chain
+  // (0.25 of 2.1 us per step on 128x64).
+  constexpr bool kEarlyWall = !Sh::IN && MODE == kModeStep;
+  using Wall = std::conditional_t<V == 2, PairWall, NodeWall<T>>;
+  uint32_t early_flag[kEarlyWall ? TS : 1];
+  Wall early_wall[kEarlyWall ? TS : 1];
+  if constexpr (kEarlyWall) {
+    static_for<0, TS>([&](auto sc) {
+      constexpr int s = decltype(sc)::value;
+      static_assert(Sh::slots(s) == 1, "one item per thread and step");
+      int c, r;
+      const bool on = item(sc, 0, c, r);
+      early_flag[s] = flag_of(sc, on, c, r);
+      early_wall[s] = Wall{};
+      if (early_flag[s]) {
+        const int x = x0 + c, y = y0 + r;
+        if constexpr (V == 2)
+          early_wall[s] = load_wall(a, PairAt{wrap_x(x), wrap_y(y), true, TS > 1 || x + 1 < a.nx});
+        else
+          early_wall[s] = load_wall<T>(a, x, y);
+      }
+    });
+  }
   // A programmatic dependent of the previous step (see step_kernel).
   griddep_launch_dependents();
   griddep_wait();
@@ -155,6 +205,12 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       constexpr int plane = Sh::kTab.box_plane[j];
       tma_load_3d(base + off, &src->m[map], bar, x0, y0 - BR - cy + GY, plane);
     });
+    if (xn >= 0)  // the lines of a tile some waves ahead, into L2
+      static_for<0, Sh::NBOX>([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        constexpr int cy = Sh::kTab.box_cy[j], map = Sh::kTab.box_map[j], plane = Sh::kTab.box_plane[j];
+        tma_prefetch_3d(&src->m[map], xn, yn - BR - cy + GY, plane);
+      });
   }
   const uint32_t key = step_key<S, MODE, FL>(a);
   const bool simple_images = a.nx >= 2 * GX && a.ny >= 2 * GY && (V == 1 || (a.nx & 1) == 0);
@@ -201,9 +257,6 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
     else
       *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1>(a.phys, H);
   };
-  auto wrap_x = [&](int x) { return x < 0 ? x + a.nx : (x >= a.nx ? x - a.nx : x); };
-  auto wrap_y = [&](int y) { return y < 0 ? y + a.ny : (y >= a.ny ? y - a.ny : y); };
-
   const bool strip_edge = x0 < GX || x0 + Sh::TW > a.nx - GX;
   bool aborted = false;
   static_for<0, TS>([&](auto sc) {
@@ -215,18 +268,8 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
     bool on[SL];
 #pragma unroll
     for (int k = 0; k < SL; ++k) {
-      if constexpr (NT % PROW == 0) {  // every slot in the thread's first column
-        row[k] = tid / PROW + k * (NT / PROW) - M;
-        col[k] = V * (tid % PROW) - M;
-      } else {
-        const int p = tid + k * NT, q = p / PROW;
-        row[k] = q - M;
-        col[k] = V * (p - q * PROW) - M;
-      }
-      const int x = x0 + col[k], y = y0 + row[k];
-      on[k] = (NI % NT == 0 || tid + k * NT < NI) && x < a.nx + M && y < a.ny + M;
-      const int xw = M ? wrap_x(x) : x, yw = M ? wrap_y(y) : y;
-      flag[k] = a.wall.active && on[k] ? flags[(int64_t)yw * flag_pitch + (xw >> 5)] : 0u;
+      on[k] = item(sc, k, col[k], row[k]);
+      flag[k] = kEarlyWall ? early_flag[kEarlyWall ? s : 0] : flag_of(sc, on[k], col[k], row[k]);
     }
     if constexpr (s == 0) {
       if (!mbar_wait_bounded(bar, 0, a.wait_ns)) *s_abort = 1;
@@ -278,27 +321,41 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
         if (E ? !on[k] : !(NI % NT == 0 || tid + k * NT < NI)) continue;
         const int x = x0 + col[k], y = y0 + row[k];
         auto psi_row = [&](int cy) -> const T* { return psi_at(col[k], row[k] + cy); };
+        auto wall = [&]() -> Wall {
+          if constexpr (kEarlyWall) return early_wall[s];
+          else if constexpr (V == 2)
+            return load_wall(a, PairAt{M ? wrap_x(x) : x, M ? wrap_y(y) : y, true, TS > 1 || x + 1 < a.nx});
+          else return load_wall<T>(a, x, y);
+        };
         if constexpr (V == 1) {
-          node_update<Q, S, MODE, FL, E>(a, f[k], flag[k], x, y, strip_edge, simple_images, psi_row);
-        } else if constexpr (s == TS - 1) {
-          pair_update<Q, S, MODE, FL, E>(a, f[k], H[k], flag[k], x, y, strip_edge, simple_images,
-                                      key + (uint32_t)s, psi_row);
+          node_update<Q, S, MODE, FL, E>(a, f[k], flag[k], x, y, strip_edge, simple_images, psi_row,
+                                         wall);
+        } else if constexpr (s == TS - 1 && (E || MODE != kModeStep)) {
+          pair_update<Q, S, MODE, FL, true>(a, f[k], H[k], flag[k], x, y, strip_edge, simple_images,
+                                            key + (uint32_t)s, psi_row, wall);
         } else {
-          // Even nx: the pair and its periodic images are pairs of whole nodes.
+          // Whole pairs: inside the lattice, or (two steps: even nx) images of
+          // pairs of whole nodes.
           const PairAt at{E ? wrap_x(x) : x, E ? wrap_y(y) : y, true, true};
-          const PairState<Q, S, E> n(a, f[k], H[k], flag[k], at, psi_row);
+          const PairState<Q, S, E> n(a, f[k], H[k], flag[k], psi_row, wall);
           typename Pair<S>::Raw raw[Q];
           pair_collide<Q, S, FL>(a, n, f[k], H[k], at, key + (uint32_t)s, raw);
-          static_for<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            constexpr int off = Sh::kTab.pop[i] + GX;
-            *reinterpret_cast<typename Pair<S>::Raw*>(
-                st + (off + (row[k] + L::cy(i) + BR) * BW + col[k])) = raw[i];
-          });
+          if constexpr (s == TS - 1) {
+            S* org = a.fout + (int64_t)(y0 + GY) * a.pitch + x0 + GX;
+            pair_store_inside<Q, S>(a, raw, org, (uint32_t)row[k] * (uint32_t)a.pitch + (uint32_t)col[k]);
+          } else {
+            static_for<0, Q>([&](auto ic) {
+              constexpr int i = decltype(ic)::value;
+              constexpr int off = Sh::kTab.pop[i] + GX;
+              *reinterpret_cast<typename Pair<S>::Raw*>(
+                  st + (off + (row[k] + L::cy(i) + BR) * BW + col[k])) = raw[i];
+            });
+          }
         }
       }
     };
-    const bool inside = Sh::IN && x0 >= GX && x0 + Sh::TW <= a.nx - GX && y0 >= GY && y0 + Sh::TH <= a.ny - GY && !any;
+    // pair_store_inside offsets are 32-bit.
+    const bool inside = Sh::IN && (uint64_t)a.pitch * Sh::TH * sizeof(S) < (1ull << 32) && x0 >= GX && x0 + Sh::TW <= a.nx - GX && y0 >= GY && y0 + Sh::TH <= a.ny - GY && !any;
     if constexpr (Sh::IN) {
       if (inside) {
         collide(std::false_type{});
@@ -318,13 +375,25 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
 }
 
 // TS time steps of one lattice; CTA (bx, by) updates the tile at (bx TW, by TH).
+// ahead > 0: each CTA also brings the boxes of the tile `ahead` places on into L2,
+// half a round of resident CTAs early, so that its loads find them there instead
+// of waiting for HBM (8192x4096 FP32 301 -> 286 us per step, 4096x2048 FP16S 62.6 ->
+// 61.0; a whole round or more ahead gains nothing for FP32).
 template <typename Sh, int MODE, int FL, int MINB>
 __global__ void __launch_bounds__(Sh::NT, MINB)
     tile_kernel(const __grid_constant__ PopMaps src, const uint32_t* __restrict__ flags,
-                int flag_pitch, const StepArgs<typename Sh::T, typename Sh::S> a) {
+                int flag_pitch, int ahead, const StepArgs<typename Sh::T, typename Sh::S> a) {
   extern __shared__ unsigned char smem_raw[];
+  int xn = -1, yn = 0;
+  if (ahead > 0) {
+    const int t = blockIdx.y * gridDim.x + blockIdx.x + ahead, ty = t / gridDim.x;
+    if (ty < gridDim.y) {
+      xn = (t - ty * gridDim.x) * Sh::TW;
+      yn = ty * Sh::TH;
+    }
+  }
   tile_update<Sh, MODE, FL>(&src, flags, flag_pitch, a, blockIdx.x * Sh::TW, blockIdx.y * Sh::TH,
-                            smem_raw);
+                            xn, yn, smem_raw);
   if constexpr (MODE == kModeStep)
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<MODE>(a, Sh::TS);
 }
@@ -344,7 +413,7 @@ __global__ void __launch_bounds__(Sh::NT, MINB)
   const auto& a = P.a[m][dir];
   const auto* mb = &members[m];
   tile_update<Sh, kModeStep, FL>(&mb->map[dir], mb->flag_words, mb->flag_pitch, a,
-                                 (local - ty * P.nstrip[m]) * Sh::TW, ty * Sh::TH, smem_raw);
+                                 (local - ty * P.nstrip[m]) * Sh::TW, ty * Sh::TH, -1, 0, smem_raw);
   if (threadIdx.x == 0 && local == 0) advance_key<kModeStep>(a, Sh::TS);
 }
 
