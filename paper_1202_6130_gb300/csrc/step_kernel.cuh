@@ -618,16 +618,17 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
   const int y0 = blockIdx.y * a.tile_rows;
   uint32_t g = 0;
   // Launched as a programmatic dependent of the previous step: the next step's
-  // CTAs may be scheduled as this grid's last wave drains; every global read
-  // or write (populations, the step counter, the status word) follows the
-  // wait for the previous grid.
-  griddep_launch_dependents();
+  // CTAs may be scheduled as this grid's last wave drains (each CTA lets them in
+  // when its march is done: earlier they pile up on the SMs, 9.6 against 8.7 us
+  // per step on 1024x512 FP32); every global read or write (populations, the step
+  // counter, the status word) follows the wait for the previous grid.
   griddep_wait();
   // Every CTA reads the counter in march_any before this launch ends; the
   // word written here is read only by the next step.
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<kModeStep>(a);
   march_any<Q, S, W, NS, FL>(&src, &flg, a, blockIdx.x * W, y0, min(a.tile_rows, a.ny - y0),
                                (blockIdx.y & 1u) != 0u, sm, g, policy);
+  griddep_launch_dependents();
 }
 
 // A lattice of a batch: TMA maps of its two population buffers for the batch's
@@ -687,7 +688,6 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
   const uint64_t policy = step_smem_init(sm);
   uint32_t g = 0;
   // A programmatic dependent of the chunk's previous step (see step_kernel).
-  griddep_launch_dependents();
   griddep_wait();
   auto march_tile = [&](int t) -> bool {
     const int m = batch_member(P, t);
@@ -711,6 +711,7 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
   } else {
     march_tile((int)blockIdx.x);
   }
+  griddep_launch_dependents();
 }
 
 }  // namespace lbm

@@ -194,9 +194,7 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       }
     });
   }
-  // A programmatic dependent of the previous step (see step_kernel).
-  griddep_launch_dependents();
-  griddep_wait();
+  griddep_wait();  // a programmatic dependent of the previous launch
   if (tid == 0) {
     mbar_arrive_expect_tx(bar, Sh::TX + a.extra_tx);
     static_for<0, Sh::NBOX>([&](auto jc) {
@@ -258,7 +256,11 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1>(a.phys, H);
   };
   const bool strip_edge = x0 < GX || x0 + Sh::TW > a.nx - GX;
-  bool aborted = false;
+  // Tiles inside the lattice: no edge, no images.
+  const bool interior = Sh::IN && x0 >= GX && x0 + Sh::TW <= a.nx - GX && y0 >= GY &&
+                        y0 + Sh::TH <= a.ny - GY &&
+                        (uint64_t)a.pitch * Sh::TH * sizeof(S) < (1ull << 32);  // 32-bit store offsets
+  bool aborted = false, inside = false;
   static_for<0, TS>([&](auto sc) {
     constexpr int s = decltype(sc)::value;
     constexpr int M = Sh::margin(s), SL = Sh::slots(s), PROW = Sh::prow(s), NI = Sh::items(s);
@@ -269,7 +271,9 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
 #pragma unroll
     for (int k = 0; k < SL; ++k) {
       on[k] = item(sc, k, col[k], row[k]);
-      flag[k] = kEarlyWall ? early_flag[kEarlyWall ? s : 0] : flag_of(sc, on[k], col[k], row[k]);
+      // A tile found inside by the first step's (larger) region stays so.
+      flag[k] = kEarlyWall ? early_flag[kEarlyWall ? s : 0]
+                           : (s > 0 && inside ? 0u : flag_of(sc, on[k], col[k], row[k]));
     }
     if constexpr (s == 0) {
       if (!mbar_wait_bounded(bar, 0, a.wait_ns)) *s_abort = 1;
@@ -303,11 +307,11 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       for (int h = NT - 1 - tid; h < 2 * NR; h += NT)
         node_psi(h < NR ? -M - 1 : Sh::TW + M, (h < NR ? h : h - NR) - M - 1);
     }
-    uint32_t any = 0;
-    if constexpr (Sh::IN) {
+    if constexpr (Sh::IN && s == 0) {
+      uint32_t any = 0;
 #pragma unroll
       for (int k = 0; k < SL; ++k) any |= flag[k];
-      any = __syncthreads_or((int)any);
+      inside = !__syncthreads_or((int)any) && interior;
     } else {
       __syncthreads();
     }
@@ -354,8 +358,6 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
         }
       }
     };
-    // pair_store_inside offsets are 32-bit.
-    const bool inside = Sh::IN && (uint64_t)a.pitch * Sh::TH * sizeof(S) < (1ull << 32) && x0 >= GX && x0 + Sh::TW <= a.nx - GX && y0 >= GY && y0 + Sh::TH <= a.ny - GY && !any;
     if constexpr (Sh::IN) {
       if (inside) {
         collide(std::false_type{});
@@ -364,6 +366,12 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
     }
     collide(std::true_type{});
   });
+  // Only now may the next launch's CTAs come: those that come while this one's
+  // still compute pile up on the SMs that are free at that moment, and several
+  // steps ahead, since each lets the next one in (GB300, us per step with the
+  // trigger at the start / here: 128x64 FP64 17 / 7.8, 400x200 FP64 43 / 30, 128x64
+  // FP32 1.85 / 1.69, D2Q21 FP32 4.4 / 3.3, 650x150 6.3 / 5.9).
+  griddep_launch_dependents();
   if (aborted && tid == 0) {
     // The boxes never arrived in full.  Record it, retire the bytes that the
     // barrier was told to expect beyond its copies (the test hook), and wait
