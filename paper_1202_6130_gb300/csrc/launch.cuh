@@ -92,17 +92,17 @@ template <int Q, typename S> constexpr TileList tile_list() {
              {64, 8, 128, 1, true, 7, 2.3, 6.6},
              {32, 4, 160, 2, false, 4, 2.0, 3.35},
              {32, 8, 224, 2, false, 3, 2.6, 3.9},
-             {32, 16, 192, 2, true, 4, 5.3, 6.0},
-             {64, 12, 288, 2, true, 3, 5.0, 6.8},
-             {64, 24, 320, 2, true, 2, 7.0, 8.3}}, 7, 0};
+             {32, 28, 288, 2, true, 3, 6.3, 7.3},
+             {64, 12, 288, 2, true, 3, 5.0, 6.6},
+             {64, 22, 448, 2, true, 2, 7.0, 7.4}}, 7, 0};
   else
     return {{{32, 4, 64, 1, false, 8, 2.2, 2.9},
-             {64, 8, 128, 1, true, 7, 3.4, 3.9},
+             {64, 8, 128, 1, true, 7, 3.0, 3.85},
              {32, 4, 160, 2, false, 4, 1.7, 3.2},
              {32, 8, 224, 2, false, 3, 2.5, 3.3},
-             {32, 16, 192, 2, true, 4, 4.7, 5.4},
-             {64, 12, 288, 2, true, 3, 4.6, 5.8},
-             {64, 24, 320, 2, true, 2, 6.7, 7.2}}, 7, 0};
+             {32, 28, 288, 2, true, 3, 4.4, 6.6},
+             {64, 12, 288, 2, true, 3, 4.5, 5.85},
+             {64, 22, 448, 2, true, 2, 5.5, 6.6}}, 7, 0};
 }
 template <int Q, typename S, int K> struct TileConfig {
   static constexpr TileCfg kCfg = tile_list<Q, S>().t[K];
