@@ -29,7 +29,7 @@ template <typename S> struct PairRho {
 // psi of both nodes of a pair.
 template <int Q, typename S, int FL>
 __device__ __forceinline__ float2 pair_psi(const Physics<float>& P, F2 rho) {
-  constexpr int kPsiKind = FL == kFlExpPlain ? 0 : -1;
+  constexpr int kPsiKind = kPsiOf<FL>;
   constexpr bool kFastExp = Codec<S>::kShifted;
   if constexpr (kPsiKind == 0 && kFastExp) {
     // psi_exp_fast of both nodes, the product and the fused multiply-add packed
@@ -241,7 +241,7 @@ __device__ __forceinline__ void pair_collide(const Args& a, const St& n, F2 (&f_
   const F2 us2 = fma2(usy, usy, usx * usx), u2 = fma2(uy, uy, ux * ux);
   const F2 wB = fma2(fma2(ngg, u2, us2), F2::splat(-T(E::inv_2theta)),
                      F2::splat(a.phys.omega));
-  if (FL != kFlExpPlain && a.phys.project) {
+  if (FL == kFlRuntime && a.phys.project) {
     // rare path: per node.  The projection is linear and maps the
     // shift w_i rho_s to itself, so it acts on h with (H, J) as it
     // acts on f with (rho, j).
@@ -309,7 +309,7 @@ __device__ __forceinline__ void pair_collide(const Args& a, const St& n, F2 (&f_
   // Round both nodes once (stochastic rounding: bits from the node pair and
   // the step).
   if constexpr (C::kShifted) {
-    if (FL == kFlExpPlain || a.stochastic) {
+    if (rounds_stochastically<FL>(a)) {
       const uint32_t h = sr_hash((uint32_t)at.x, (uint32_t)at.y, key);
       static_for<0, Q>([&](auto ic) {
         constexpr int i = decltype(ic)::value;
@@ -510,7 +510,7 @@ __device__ __forceinline__ void node_update(const Args& a, T (&f)[Q], uint32_t f
     if constexpr (MODE == kModeStep) {
       const T usx = ux + div_rho<T>(Fx, rho, inv_rho);
       const T usy = uy + div_rho<T>(Fy, rho, inv_rho);
-      if (FL != kFlExpPlain && a.phys.project) project<Q, T>(f, rho, jx, jy);
+      if (FL == kFlRuntime && a.phys.project) project<Q, T>(f, rho, jx, jy);
       node_collide<Q, T>(a.phys, f, rho, ux, uy, usx, usy);
       // The primary store plus periodic images inside the ghost frame.
       S e[Q];

@@ -125,6 +125,9 @@ cudaError_t launch_tile(int shape, const PopMaps& src, const uint32_t* flags, in
     return launch_tile_k<Q, S, tile_list<Q, S>().moments, kModeMoments, kFlRuntime>(
         src, flags, flag_pitch, a, stream);
   return with_shape<Q, S>(shape, [&]<int K>() {
+    if constexpr (Q == 9 && sizeof(S) == 2)
+      if (a.phys.psi_kind == 0 && !a.phys.project && !a.stochastic)
+        return launch_tile_k<Q, S, K, kModeStep, kFlExpNearest>(src, flags, flag_pitch, a, stream);
     return plain_flags(a) ? launch_tile_k<Q, S, K, kModeStep, kFlExpPlain>(src, flags, flag_pitch, a, stream)
                           : launch_tile_k<Q, S, K, kModeStep, kFlRuntime>(src, flags, flag_pitch, a, stream);
   });

@@ -195,7 +195,7 @@ __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensor
   using T = typename Codec<S>::T;
   using C = Codec<S>;
   static_assert(!C::kShifted, "16-bit storage runs the paired march");
-  constexpr int kPsiKind = FL == kFlExpPlain ? 0 : -1;
+  constexpr int kPsiKind = kPsiOf<FL>;
   constexpr int R = Sh::R;
   constexpr int GX = Sh::GX;
   constexpr int GY = Sh::GY;
@@ -395,7 +395,7 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
   constexpr int P = Sh::V / 2;  // node pairs per thread
   constexpr bool kRegs = Sh::kRegs;
   static_assert(Sh::V % 2 == 0 && RO % 2 == 0 && RO >= R, "paired march");
-  constexpr int kPsiKind = FL == kFlExpPlain ? 0 : -1;
+  constexpr int kPsiKind = kPsiOf<FL>;
   constexpr bool kFastExp = C::kShifted;
   unsigned char* const stages = sm.stages;
   uint64_t* const bars = sm.bars;

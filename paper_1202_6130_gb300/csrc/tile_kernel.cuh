@@ -228,10 +228,10 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       H = (decltype(ic)::value == 0) ? v : H + v;
     });
     if constexpr (V == 2)
-      *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1, C::kShifted>(
+      *psi_at(c, r) = pseudo_potential<Q, T, kPsiOf<FL>, C::kShifted>(
           a.phys, PairRho<S>::of(a.phys, H));
     else
-      *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1>(a.phys, H);
+      *psi_at(c, r) = pseudo_potential<Q, T, kPsiOf<FL>>(a.phys, H);
   };
   // Loads the item at (c, r) (a node pair or a node) into f, its sum into H,
   // and forms its psi.
@@ -253,7 +253,7 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       *reinterpret_cast<float2*>(psi_at(c, r)) =
           pair_psi<Q, S, FL>(a.phys, PairRho<S>::of(a.phys, H));
     else
-      *psi_at(c, r) = pseudo_potential<Q, T, FL == kFlExpPlain ? 0 : -1>(a.phys, H);
+      *psi_at(c, r) = pseudo_potential<Q, T, kPsiOf<FL>>(a.phys, H);
   };
   const bool strip_edge = x0 < GX || x0 + Sh::TW > a.nx - GX;
   // Tiles inside the lattice: no edge, no images.
