@@ -42,10 +42,10 @@ DTYPE = {"fp64": "f64", "fp32": "f32", "fp16s": "f16", "bf16s": "bf16"}
 BYTES = {"fp64": 8, "fp32": 4, "fp16s": 2, "bf16s": 2}
 # FP64 storage is bound by the FP64 pipe, not by HBM.  Its roofline counts the
 # FP64 flops the step executes per node update (2 x DFMA + DADD + DMUL, ncu on
-# 4096x2048; about 2% of them are the recomputed halo psi) against the DFMA
+# 2048x1024; about 5% of them are the recomputed halo psi) against the DFMA
 # peak: SMs x 2 DFMA per cycle x 2 flops x SM clock (GB300: 152 x 2 x 2 x
 # 2.07 GHz = 1.26 TFLOP/s, its nominal FP64 rate).
-FP64_FLOPS_PER_NODE = {9: 288, 21: 514}
+FP64_FLOPS_PER_NODE = {9: 188, 21: 351}
 FP64_DFMA_PER_SM_CLK = 2
 
 
