@@ -97,9 +97,10 @@ static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int 
   cudaError_t e = prepare_tile<Q, S, K, MODE, FL>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW, (a.ny + Sh::TH - 1) / Sh::TH);
+  const int nty = (a.ny + Sh::TH - 1) / Sh::TH, gy = nty < 65535 ? nty : 65535;
+  cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW, gy, (nty + gy - 1) / gy);
   const int slots = Sh::IN ? tile_slots<Q, S, K>() : 0;
-  const int ahead = (int64_t)cfg.gridDim.x * cfg.gridDim.y > slots ? slots / 2 : 0;
+  const int ahead = (int64_t)cfg.gridDim.x * nty > slots ? slots / 2 : 0;
   cfg.blockDim = dim3(Sh::NT);
   cfg.dynamicSmemBytes = Sh::SMEM;
   cfg.stream = stream;

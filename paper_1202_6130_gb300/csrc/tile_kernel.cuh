@@ -382,7 +382,7 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
   }
 }
 
-// TS time steps of one lattice; CTA (bx, by) updates the tile at (bx TW, by TH).
+// TS time steps of one lattice, one CTA per tile.
 // ahead > 0: each CTA also brings the boxes of the tile `ahead` places on into L2,
 // half a round of resident CTAs early, so that its loads find them there instead
 // of waiting for HBM (8192x4096 FP32 301 -> 286 us per step, 4096x2048 FP16S 62.6 ->
@@ -392,18 +392,21 @@ __global__ void __launch_bounds__(Sh::NT, MINB)
     tile_kernel(const __grid_constant__ PopMaps src, const uint32_t* __restrict__ flags,
                 int flag_pitch, int ahead, const StepArgs<typename Sh::T, typename Sh::S> a) {
   extern __shared__ unsigned char smem_raw[];
+  // Tile rows beyond the 65,535 of a grid's y go on in z.
+  const int ty = blockIdx.z * gridDim.y + blockIdx.y;
+  if (ty * Sh::TH >= a.ny) return;
   int xn = -1, yn = 0;
   if (ahead > 0) {
-    const int t = blockIdx.y * gridDim.x + blockIdx.x + ahead, ty = t / gridDim.x;
-    if (ty < gridDim.y) {
-      xn = (t - ty * gridDim.x) * Sh::TW;
-      yn = ty * Sh::TH;
+    const int next = ty * gridDim.x + blockIdx.x + ahead, tn = next / gridDim.x;
+    if (tn * Sh::TH < a.ny) {
+      xn = (next - tn * gridDim.x) * Sh::TW;
+      yn = tn * Sh::TH;
     }
   }
-  tile_update<Sh, MODE, FL>(&src, flags, flag_pitch, a, blockIdx.x * Sh::TW, blockIdx.y * Sh::TH,
-                            xn, yn, smem_raw);
+  tile_update<Sh, MODE, FL>(&src, flags, flag_pitch, a, blockIdx.x * Sh::TW, ty * Sh::TH, xn, yn,
+                            smem_raw);
   if constexpr (MODE == kModeStep)
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<MODE>(a, Sh::TS);
+    if (blockIdx.x == 0 && ty == 0 && threadIdx.x == 0) advance_key<MODE>(a, Sh::TS);
 }
 
 // One step of up to kChunk lattices of a batch on tiles: CTA b updates tile b of

@@ -75,7 +75,8 @@ def footprint_bytes(nx: int, ny: int, storage: str, lattice: int = 9) -> int:
     r = 1 if lattice == 9 else 3
     gx = ((2 * r * s + 15) // 16) * 16 // s
     pitch = ((nx + 2 * gx + 31) // 32) * 32
-    pops = 2 * lattice * pitch * (ny + 4 * r) * s
+    gy = 4 if lattice == 9 else 6  # ghost rows above and below
+    pops = 2 * lattice * pitch * (ny + 2 * gy) * s
     t = 8 if storage == "fp64" else 4
     wall = 5 * nx * ny * t + ((nx + 31) // 32 + 3) // 4 * 4 * ny * 4
     staging = (lattice + 3) * nx * ny * 8

@@ -78,6 +78,23 @@ def test_one_step_tiles_equal_the_row_march_bitwise(pkg, lattice, storage, size)
     np.testing.assert_array_equal(_run(pkg, w, storage, 0, (3,))[0], _run(pkg, w, storage, 4, (3,))[0])
 
 
+def test_more_tile_rows_than_a_grid_holds(pkg):
+    """270,000 rows: 67,500 tiles of 4 rows in one column, beyond a grid's 65,535
+    in y.  The read-out (tiles of 4 rows) and two steps equal the row march."""
+    nx, ny = 8, 270000
+    rho = 1.0 + 0.1 * W.uniform(5, nx * ny, -1.0, 1.0).reshape(ny, nx)
+    out = []
+    for tile_rows in (0, 8):
+        sim = pkg.Simulation(nx, ny, storage="fp16s", tile_rows=tile_rows, shift_rho=1.0)
+        sim.set_equilibrium(rho)
+        r0 = sim.moments()[0]
+        assert np.abs(r0 - rho).max() < 1e-3
+        sim.step(3)
+        out.append(sim.populations())
+        sim.close()
+    np.testing.assert_array_equal(out[0], out[1])
+
+
 def test_checks_fall_between_the_steps_of_two(pkg):
     """check_every = 3 reports a non-finite density on the step it is due (the
     state stays as after that step), although two steps fit one launch."""
