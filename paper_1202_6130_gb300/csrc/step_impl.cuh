@@ -2,6 +2,8 @@
 // storage type, which instantiates them for D2Q9 and D2Q21.
 #pragma once
 
+#include <algorithm>
+
 #include "launch.cuh"
 
 namespace lbm {
@@ -97,8 +99,8 @@ static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int 
   cudaError_t e = prepare_tile<Q, S, K, MODE, FL>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  const int nty = (a.ny + Sh::TH - 1) / Sh::TH, gy = nty < 65535 ? nty : 65535;
-  cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW, gy, (nty + gy - 1) / gy);
+  const int nty = (a.ny + Sh::TH - 1) / Sh::TH;
+  cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW);
   const int slots = Sh::IN ? tile_slots<Q, S, K>() : 0;
   const int ahead = (int64_t)cfg.gridDim.x * nty > slots ? slots / 2 : 0;
   cfg.blockDim = dim3(Sh::NT);
@@ -109,7 +111,11 @@ static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tile_kernel<Sh, MODE, FL, Cfg::kCfg.minb>, src, flags, flag_pitch, ahead, a);
+  for (int ty0 = 0; ty0 < nty && e == cudaSuccess; ty0 += 65535) {
+    cfg.gridDim.y = std::min(nty - ty0, 65535);
+    e = cudaLaunchKernelEx(&cfg, tile_kernel<Sh, MODE, FL, Cfg::kCfg.minb>, src, flags, flag_pitch, ahead, ty0, a);
+  }
+  return e;
 }
 
 // Calls fn<K>() for the K-th shape of the list.

@@ -382,7 +382,8 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
   }
 }
 
-// TS time steps of one lattice, one CTA per tile.
+// TS time steps of one lattice, one CTA per tile; ty0: the launch's first row of
+// tiles (a grid holds 65,535 of them, taller lattices take several launches).
 // ahead > 0: each CTA also brings the boxes of the tile `ahead` places on into L2,
 // half a round of resident CTAs early, so that its loads find them there instead
 // of waiting for HBM (8192x4096 FP32 301 -> 286 us per step, 4096x2048 FP16S 62.6 ->
@@ -390,11 +391,9 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
 template <typename Sh, int MODE, int FL, int MINB>
 __global__ void __launch_bounds__(Sh::NT, MINB)
     tile_kernel(const __grid_constant__ PopMaps src, const uint32_t* __restrict__ flags,
-                int flag_pitch, int ahead, const StepArgs<typename Sh::T, typename Sh::S> a) {
+                int flag_pitch, int ahead, int ty0, const StepArgs<typename Sh::T, typename Sh::S> a) {
   extern __shared__ unsigned char smem_raw[];
-  // Tile rows beyond the 65,535 of a grid's y go on in z.
-  const int ty = blockIdx.z * gridDim.y + blockIdx.y;
-  if (ty * Sh::TH >= a.ny) return;
+  const int ty = blockIdx.y + ty0;
   int xn = -1, yn = 0;
   if (ahead > 0) {
     const int next = ty * gridDim.x + blockIdx.x + ahead, tn = next / gridDim.x;
