@@ -300,7 +300,8 @@ int lbm_batch_set_tiling(lbm_batch* b, int32_t tile_rows, int32_t ctas);
 /* Advances every member by nsteps time steps; enqueued on the batch stream. */
 int lbm_batch_step(lbm_batch* b, int64_t nsteps);
 /* Times each candidate tiling (the default tiles; row marches of 4..64 rows x
- * {one CTA per segment, one persistent wave}) for steps_per_trial steps (plus 18 warm-up steps) on the members
+ * {one CTA per segment, one persistent wave}; 14 trials) for steps_per_trial
+ * steps (plus 18 warm-up steps) on the members
  * themselves -- so they advance by those steps -- keeps the fastest, and
  * records it for the batch's size class (see lbm_batch_use_tuned).
  * best_tile_rows is the chosen tiling's rows per CTA.  Outputs may be NULL.  Synchronises the stream. */
