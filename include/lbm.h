@@ -263,8 +263,8 @@ int lbm_wall_core_tail(int32_t nx, int32_t ny, const double* dist, const double*
 /* ---- batches: many lattices advanced by shared launches --------------------- */
 
 /* A batch advances several contexts (its members) together: every time step is
- * one launch of one fused kernel per chunk of up to 64 members (32 with FP64
- * storage), whose CTAs march
+ * one launch of one fused kernel per chunk of up to 64 members (40 for D2Q21, 32
+ * with FP64 storage), whose CTAs march
  * the chunk's (member, strip, segment) tiles, each launched as a programmatic
  * dependent of the chunk's previous step; the chunks run on streams forked
  * from the batch stream, and runs of 16 and of 2 consecutive steps are
@@ -275,8 +275,9 @@ int lbm_wall_core_tail(int32_t nx, int32_t ny, const double* dist, const double*
  * memory, and can still be read with lbm_moments and friends between batch
  * steps.  Stepping a member on its own, or changing its wall or stream,
  * between batch steps is allowed; the batch notices and rebuilds its tile
- * list.  The batch's own small descriptor arrays come from a (nullable)
- * allocator.  Graph capture needs a non-default stream; with a NULL stream
+ * list.  A batch holds no device memory of its own (its descriptors travel as
+ * kernel parameters); a non-null allocator is checked and not used.  Graph
+ * capture needs a non-default stream; with a NULL stream
  * every step is a plain launch.  lbm_batch_step orders itself with the
  * members' own streams by events: it starts after work already enqueued on
  * them, and work enqueued on them afterwards waits for it.  Errors are
@@ -288,8 +289,8 @@ int lbm_batch_add(lbm_batch* b, lbm_ctx* c);
 int lbm_batch_remove(lbm_batch* b, lbm_ctx* c);
 int lbm_batch_size(const lbm_batch* b, int32_t* n);
 /* Kernel launches per batch time step: the number of member chunks (members
- * divided by 64, or by 32 with FP64 storage, rounded up; 0 for an empty
- * batch). */
+ * divided by 64, by 40 for D2Q21 or by 32 with FP64 storage, rounded up; 0 for
+ * an empty batch). */
 int lbm_batch_launches_per_step(const lbm_batch* b, int32_t* n);
 /* Tiling: with both 0 (the default) the engine picks two-dimensional tiles, one
  * CTA per tile, or row marches for all members by their sizes.  tile_rows > 0 asks for row

@@ -12,6 +12,7 @@
 #include <string>
 #include <initializer_list>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <tuple>
 #include <vector>
@@ -538,7 +539,7 @@ int lbm_set_wall(lbm_ctx* c, const double* phi_s, const double* psi_r, const dou
   if (!c->wall_phie) {
     // one uint32 flag per (row, 32-column chunk); rows padded to 16 bytes so
     // that each strip's flag words are one aligned TMA box
-    c->nchunk_pad = ((nx + 31) / 32 + 3) / 4 * 4;
+    c->nchunk_pad = flag_words_per_row(nx);
     c->wall_phie = dalloc(c, N * tsz);
     c->wall_sx = dalloc(c, N * tsz);
     c->wall_sy = dalloc(c, N * tsz);
@@ -942,8 +943,6 @@ constexpr int kLongSteps = 16;
 static_assert(kLongSteps % 2 == 0, "a replay must end on the parity it started from");
 
 struct lbm_batch {
-  lbm_allocator alloc{};
-  bool user_alloc = false;
   cudaStream_t stream = nullptr;
   std::vector<lbm_ctx*> members;
   std::vector<uint64_t> versions;
@@ -953,19 +952,16 @@ struct lbm_batch {
   int ctas = 0;       // 0: one CTA per tile; > 0: row march by that many persistent CTAs
   int shape = -1;     // tile shape of the members' kernel (-1: the row march)
   bool dirty = true;
-  void* d_members = nullptr;
-  size_t cap_members = 0;
-  int ntiles = 0, nctas = 0;
   int64_t phase = 0;
   cudaGraphExec_t gexec = nullptr;       // two steps
   cudaGraphExec_t gexec_long = nullptr;  // kLongSteps steps
   cudaEvent_t order_ev = nullptr;  // orders member streams with the batch stream
   // Members are launched in chunks of up to BatchArgs::kChunk, each with its step
-  // arguments as a kernel parameter.  With several chunks every chunk has its
+  // arguments and tensor maps as a kernel parameter.  With several chunks every chunk has its
   // own stream, forked from and joined back to the batch stream around each
   // sequence of steps (a member depends only on its own previous step).
   struct Chunk {
-    std::vector<unsigned char> args;  // host copy of BatchArgs<T, S>
+    std::shared_ptr<void> args[2];    // BatchArgs<Q, T, S> of the steps at parity 0 and 1
     int base = 0, count = 0;          // members [base, base + count)
     int nctas = 0;
     bool plain = false;               // every member: exponential psi, no projection, SR
@@ -1001,37 +997,6 @@ int bfail(lbm_batch* b, int code, const char* fmt, ...) {
     if (e_ != cudaSuccess)                                                             \
       return bfail((b), LBM_ECUDA, "%s failed: %s", #__VA_ARGS__, cudaGetErrorString(e_)); \
   } while (0)
-
-void* balloc(lbm_batch* b, size_t bytes) {
-  bytes = (bytes + 255) & ~size_t(255);
-  void* p = nullptr;
-  if (b->user_alloc)
-    p = b->alloc.alloc(bytes, b->alloc.user);
-  else if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    p = nullptr;
-  }
-  return p;
-}
-
-void bfree(lbm_batch* b, void* p) {
-  if (!p) return;
-  if (b->user_alloc)
-    b->alloc.free(p, b->alloc.user);
-  else
-    cudaFree(p);
-}
-
-int bgrow(lbm_batch* b, void** p, size_t* cap, size_t need) {
-  if (*cap >= need && *p) return LBM_OK;
-  if (*p) {
-    cudaStreamSynchronize(b->stream);
-    bfree(b, *p);
-  }
-  *p = balloc(b, need);
-  *cap = *p ? need : 0;
-  return *p ? LBM_OK : bfail(b, LBM_ENOMEM, "batch descriptor of %zu bytes", need);
-}
 
 void drop_graph(lbm_batch* b) {
   if (b->gexec) {
@@ -1088,21 +1053,17 @@ template <int Q, typename S> int batch_shape(const lbm_batch* b, int* rows) {
 
 template <int Q, typename S> int batch_build(lbm_batch* b) {
   using T = typename Codec<S>::T;
-  using M = BatchMember<T, S>;
-  using A = BatchArgs<T, S>;
+  using A = BatchArgs<Q, T, S>;
   constexpr int W = StepConfig<Q, S>::W;
   const int n = (int)b->members.size();
   constexpr int kChunk = A::kChunk;
   const int nchunk = (n + kChunk - 1) / kChunk;
-  std::vector<M> hm(n);
   int rows = b->tile_rows;
   b->shape = b->tile_rows == 0 && b->ctas == 0 ? batch_shape<Q, S>(b, &rows) : -1;
   b->versions.assign(n, 0);
   b->cur0.assign(n, 0);
   for (int i = 0; i < n; ++i) {
     lbm_ctx* c = b->members[i];
-    M& m = hm[i];
-    std::memset(&m, 0, sizeof m);
     if (b->shape >= 0) {
       if (c->shape[lbm_ctx::kBatch] != b->shape) {
         c->shape[lbm_ctx::kBatch] = b->shape;
@@ -1110,10 +1071,6 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
       }
       if (ready_tile_maps<Q, S>(c, lbm_ctx::kBatch)) return bfail(b, LBM_ECUDA, "%s", c->err.c_str());
     }
-    for (int d = 0; d < 2; ++d) m.map[d] = b->shape >= 0 ? c->tile_map[lbm_ctx::kBatch][d] : c->tmap[d];
-    m.flag_words = c->wall_flags;
-    m.flag_pitch = c->nchunk_pad;
-    m.flags = c->has_wall ? c->flag_map : c->tmap[0].m[0];
     b->versions[i] = c->version;
     b->cur0[i] = c->cur;
   }
@@ -1128,39 +1085,49 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
     lbm_batch::Chunk& ch = b->chunks[k];
     ch.base = k * kChunk;
     ch.count = std::min(kChunk, n - ch.base);
-    ch.args.assign(sizeof(A), 0);
-    A* pa = reinterpret_cast<A*>(ch.args.data());
+    A* pa[2];
+    for (int parity = 0; parity < 2; ++parity) {
+      auto args = std::make_shared<A>();
+      pa[parity] = args.get();
+      ch.args[parity] = std::move(args);
+    }
     ch.plain = true;
     int32_t t0 = 0;
     for (int i = 0; i < ch.count; ++i) {
       lbm_ctx* c = b->members[ch.base + i];
       ch.plain = ch.plain && c->p.psi_kind == LBM_PSI_EXP && !c->p.project &&
                  (!Codec<S>::kShifted || c->p.rounding == LBM_ROUND_STOCHASTIC);
-      for (int d = 0; d < 2; ++d)
-        pa->a[i][d] = make_args<Q, S>(c, d, static_cast<S*>(c->buf[d ^ 1]), nullptr, nullptr, nullptr, 0);
-      pa->cur[i] = c->cur;
+      // Tiles, or march segments of about L rows, balanced over the member's
+      // height: a short remainder segment would pay its 2R halo rows and its
+      // pipeline fill for a few rows only.
+      int nseg, nstrip;
       if (b->shape >= 0) {
         const TileCfg t = tile_list<Q, S>().t[b->shape];
-        pa->nseg[i] = (c->p.ny + t.th - 1) / t.th;
-        pa->nstrip[i] = (c->p.nx + t.tw - 1) / t.tw;
-        pa->tile0[i] = t0;
-        t0 += pa->nseg[i] * pa->nstrip[i];
-        continue;
+        nseg = (c->p.ny + t.th - 1) / t.th;
+        nstrip = (c->p.nx + t.tw - 1) / t.tw;
+      } else {
+        const int L = std::max(1, std::min(rows > 0 ? rows : c->tile_rows, c->p.ny));
+        nseg = std::max(1, (c->p.ny + L / 2) / L);
+        nstrip = (c->p.nx + W - 1) / W;
       }
-      // Segments of about L rows, balanced over the member's height: a short
-      // remainder segment would pay its 2R halo rows and its pipeline fill
-      // for a few rows only.
-      const int L = std::max(1, std::min(rows > 0 ? rows : c->tile_rows, c->p.ny));
-      pa->nseg[i] = std::max(1, (c->p.ny + L / 2) / L);
-      pa->nstrip[i] = (c->p.nx + W - 1) / W;
-      pa->tile0[i] = t0;
-      t0 += pa->nseg[i] * pa->nstrip[i];
+      for (int parity = 0; parity < 2; ++parity) {
+        const int d = c->cur ^ parity;  // the buffer read
+        const PopMaps& maps = b->shape >= 0 ? c->tile_map[lbm_ctx::kBatch][d] : c->tmap[d];
+        std::copy_n(maps.m, kMapsOf<Q>, pa[parity]->map[i]);
+        pa[parity]->flags[i] = c->has_wall ? c->flag_map : maps.m[0];
+        pa[parity]->flag_words[i] = c->wall_flags;
+        pa[parity]->a[i] = make_args<Q, S>(c, d, static_cast<S*>(c->buf[d ^ 1]), nullptr, nullptr, nullptr, 0);
+        pa[parity]->tile0[i] = t0;
+        pa[parity]->nseg[i] = nseg;
+        pa[parity]->nstrip[i] = nstrip;
+      }
+      t0 += nseg * nstrip;
     }
-    for (int i = ch.count; i <= kChunk; ++i) pa->tile0[i] = t0;
+    for (A* p : pa)
+      for (int i = ch.count; i <= kChunk; ++i) p->tile0[i] = t0;
     chunk_tiles[k] = t0;
     total += (size_t)t0;
   }
-  b->nctas = 0;
   for (int k = 0; k < nchunk; ++k) {
     lbm_batch::Chunk& ch = b->chunks[k];
     // Persistent CTAs: the batch's count shared out by tiles; CTA j of a
@@ -1170,21 +1137,16 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
                    : (int)std::max<int64_t>(
                          1, std::min<int64_t>(chunk_tiles[k],
                                               std::llround((double)b->ctas * chunk_tiles[k] / total)));
-    b->nctas += ch.nctas;
     if (nchunk > 1 && !ch.stream) {
       BCK(b, cudaStreamCreateWithFlags(&ch.stream, cudaStreamNonBlocking));
       BCK(b, cudaEventCreateWithFlags(&ch.done, cudaEventDisableTiming));
     }
   }
   if (nchunk > 1 && !b->fork_ev) BCK(b, cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming));
-  b->ntiles = (int)total;
   // The kernels' shared-memory attributes, outside any capture.
   if (b->shape >= 0) BCK(b, prepare_batch_tiles<Q, S>(b->shape));
   else batch_ctas_per_sm<Q, S>();
-  int rc = bgrow(b, &b->d_members, &b->cap_members, sizeof(M) * std::max(1, n));
-  if (rc) return rc;
-  BCK(b, cudaMemcpyAsync(b->d_members, hm.data(), sizeof(M) * n, cudaMemcpyHostToDevice, b->stream));
-  BCK(b, cudaStreamSynchronize(b->stream));  // host vectors go out of scope
+  BCK(b, cudaStreamSynchronize(b->stream));  // replays of the graphs dropped below are over
   b->phase = 0;
   drop_graph(b);
   b->dirty = false;
@@ -1197,13 +1159,12 @@ template <int Q, typename S> cudaError_t batch_launch(lbm_batch* b, int parity) 
   using T = typename Codec<S>::T;
   const bool multi = b->chunks.size() > 1;
   for (const lbm_batch::Chunk& ch : b->chunks) {
-    const auto& args = *reinterpret_cast<const BatchArgs<T, S>*>(ch.args.data());
-    const auto* members = static_cast<const BatchMember<T, S>*>(b->d_members) + ch.base;
+    const auto& args = *static_cast<const BatchArgs<Q, T, S>*>(ch.args[parity].get());
     const cudaStream_t st = multi ? ch.stream : b->stream;
     const cudaError_t e =
         b->shape >= 0
-            ? launch_batch_tiles<Q, S>(b->shape, args, members, ch.nctas, parity, ch.plain, st)
-            : launch_batch<Q, S>(args, members, ch.nctas, parity, b->ctas > 0, ch.plain, st);
+            ? launch_batch_tiles<Q, S>(b->shape, args, ch.nctas, ch.plain, st)
+            : launch_batch<Q, S>(args, ch.nctas, b->ctas > 0, ch.plain, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1245,10 +1206,6 @@ int lbm_batch_create(const lbm_allocator* a, void* cuda_stream, lbm_batch** out)
   if (a && (!a->alloc || !a->free)) return bfail(nullptr, LBM_EINVAL, "allocator without alloc/free");
   lbm_batch* b = new (std::nothrow) lbm_batch();
   if (!b) return bfail(nullptr, LBM_ENOMEM, "host allocation");
-  if (a) {
-    b->alloc = *a;
-    b->user_alloc = true;
-  }
   b->stream = static_cast<cudaStream_t>(cuda_stream);
   *out = b;
   return LBM_OK;
@@ -1290,7 +1247,9 @@ int lbm_batch_size(const lbm_batch* b, int32_t* n) {
 
 int lbm_batch_launches_per_step(const lbm_batch* b, int32_t* n) {
   if (!b || !n) return bfail(nullptr, LBM_EINVAL, "null argument");
-  const int chunk = b->storage == LBM_FP64 ? batch_chunk<double>() : batch_chunk<float>();
+  const int chunk = b->storage == LBM_FP64 ? batch_chunk<9, double>()
+                    : b->Q == 9            ? batch_chunk<9, float>()
+                                           : batch_chunk<21, float>();
   *n = (int32_t)((b->members.size() + chunk - 1) / chunk);
   return LBM_OK;
 }
@@ -1535,7 +1494,6 @@ int lbm_batch_destroy(lbm_batch* b) {
   for (lbm_batch::Chunk& ch : b->chunks) release_chunk(ch);
   if (b->fork_ev) cudaEventDestroy(b->fork_ev);
   if (b->order_ev) cudaEventDestroy(b->order_ev);
-  bfree(b, b->d_members);
   delete b;
   return LBM_OK;
 }

@@ -131,16 +131,14 @@ template <int Q, typename S> int step_ctas_per_sm();
 // exponential psi, no projection and (16-bit storage) stochastic rounding, so
 // the kernel with those settings fixed runs.
 template <int Q, typename S>
-cudaError_t launch_batch(const BatchArgs<typename Codec<S>::T, S>& args,
-                         const BatchMember<typename Codec<S>::T, S>* members, int nctas,
-                         int parity, bool persistent, bool plain, cudaStream_t stream);
+cudaError_t launch_batch(const BatchArgs<Q, typename Codec<S>::T, S>& args, int nctas,
+                         bool persistent, bool plain, cudaStream_t stream);
 template <int Q, typename S> int batch_ctas_per_sm();
 
 // The same on tiles of shape `shape`, one CTA per tile.
 template <int Q, typename S>
-cudaError_t launch_batch_tiles(int shape, const BatchArgs<typename Codec<S>::T, S>& args,
-                               const BatchMember<typename Codec<S>::T, S>* members, int ntiles,
-                               int parity, bool plain, cudaStream_t stream);
+cudaError_t launch_batch_tiles(int shape, const BatchArgs<Q, typename Codec<S>::T, S>& args,
+                               int ntiles, bool plain, cudaStream_t stream);
 // Sets the shared-memory attribute of its kernels (outside any stream capture).
 template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape);
 

@@ -24,7 +24,10 @@ enum StepMode : int {
 enum StepFlags : int { kFlRuntime = 0, kFlExpPlain = 1, kFlExpNearest = 2 };
 template <int FL> constexpr int kPsiOf = FL == kFlRuntime ? -1 : 0;  // psi kind, -1: P.psi_kind
 
-template <typename T, typename S> struct StepArgs {
+// Wall-flag words per lattice row: one per 32 columns, padded to 16 bytes.
+__host__ __device__ constexpr int flag_words_per_row(int nx) { return ((nx + 31) / 32 + 3) / 4 * 4; }
+
+template <typename T, typename S> struct StepCore {
   Physics<T> phys;
   WallFields<T> wall;
   int32_t nx, ny;
@@ -32,10 +35,6 @@ template <typename T, typename S> struct StepArgs {
   int32_t tile_rows;   // L
   int64_t plane;       // elements per population plane
   S* fout;             // kModeStep: destination buffer (same layout as the source)
-  double* out_rho;     // kModeMoments: [ny][nx]
-  double* out_ux;
-  double* out_uy;
-  int32_t momentum;    // kModeMoments: 1 -> out_ux/out_uy get j + F/2 instead of u
   uint32_t* status;    // error bits (kStatus*)
   uint64_t wait_ns;    // bound of every stage wait
   uint32_t extra_tx;   // test hook: bytes each stage expects beyond its copies (0 normally)
@@ -45,6 +44,12 @@ template <typename T, typename S> struct StepArgs {
   uint32_t* rng;
   int32_t rng_idx;
   int32_t stochastic;  // 16-bit storage: 1 = stochastic rounding, 0 = nearest-even
+};
+template <typename T, typename S> struct StepArgs : StepCore<T, S> {
+  double* out_rho;     // kModeMoments: [ny][nx]
+  double* out_ux;
+  double* out_uy;
+  int32_t momentum;    // kModeMoments: 1 -> out_ux/out_uy get j + F/2 instead of u
 };
 
 template <int FL, typename Args> __device__ __forceinline__ bool rounds_stochastically(const Args& a) {
@@ -69,6 +74,7 @@ __device__ __forceinline__ void advance_key(const Args& a, uint32_t steps = 1u) 
 // TMA maps of one population buffer, one per distinct box depth of the
 // lattice's plane groups (D2Q9 uses one, D2Q21 three).
 constexpr int kMaxMaps = 3;
+template <int Q> constexpr int kMapsOf = Q == 9 ? 1 : kMaxMaps;
 struct PopMaps {
   CUtensorMap m[kMaxMaps];
 };

@@ -180,9 +180,8 @@ static cudaError_t prepare_batch_kernel() {
 }
 
 template <int Q, typename S, int FL>
-static cudaError_t launch_batch_fl(const BatchArgs<typename Codec<S>::T, S>& args,
-                                   const BatchMember<typename Codec<S>::T, S>* members,
-                                   int nctas, int parity, bool persistent, cudaStream_t stream) {
+static cudaError_t launch_batch_fl(const BatchArgs<Q, typename Codec<S>::T, S>& args, int nctas,
+                                   bool persistent, cudaStream_t stream) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
   cudaError_t e = prepare_batch_kernel<Q, S, FL>();
@@ -200,17 +199,16 @@ static cudaError_t launch_batch_fl(const BatchArgs<typename Codec<S>::T, S>& arg
   cfg.numAttrs = 1;
   if (persistent)
     return cudaLaunchKernelEx(&cfg, batch_step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::BATCH_MINB, true, FL>,
-                              args, members, parity);
+                              args);
   return cudaLaunchKernelEx(&cfg, batch_step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::template batch_minb_tile<FL>(), false, FL>,
-                            args, members, parity);
+                            args);
 }
 
 template <int Q, typename S>
-cudaError_t launch_batch(const BatchArgs<typename Codec<S>::T, S>& args,
-                         const BatchMember<typename Codec<S>::T, S>* members, int nctas,
-                         int parity, bool persistent, bool plain, cudaStream_t stream) {
-  return plain ? launch_batch_fl<Q, S, kFlExpPlain>(args, members, nctas, parity, persistent, stream)
-               : launch_batch_fl<Q, S, kFlRuntime>(args, members, nctas, parity, persistent, stream);
+cudaError_t launch_batch(const BatchArgs<Q, typename Codec<S>::T, S>& args, int nctas,
+                         bool persistent, bool plain, cudaStream_t stream) {
+  return plain ? launch_batch_fl<Q, S, kFlExpPlain>(args, nctas, persistent, stream)
+               : launch_batch_fl<Q, S, kFlRuntime>(args, nctas, persistent, stream);
 }
 
 // Residency per SM of the persistent batch kernel; also sets the shared-memory
@@ -247,9 +245,8 @@ template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape) {
 }
 
 template <int Q, typename S>
-cudaError_t launch_batch_tiles(int shape, const BatchArgs<typename Codec<S>::T, S>& args,
-                               const BatchMember<typename Codec<S>::T, S>* members, int ntiles,
-                               int parity, bool plain, cudaStream_t stream) {
+cudaError_t launch_batch_tiles(int shape, const BatchArgs<Q, typename Codec<S>::T, S>& args,
+                               int ntiles, bool plain, cudaStream_t stream) {
   return with_shape<Q, S>(shape, [&]<int K>() {
     using Cfg = TileConfig<Q, S, K>;
     using Sh = typename Cfg::Sh;
@@ -266,8 +263,8 @@ cudaError_t launch_batch_tiles(int shape, const BatchArgs<typename Codec<S>::T, 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return plain ? cudaLaunchKernelEx(&cfg, batch_tile_kernel<Sh, kFlExpPlain, Cfg::kCfg.minb>, args, members, parity)
-                 : cudaLaunchKernelEx(&cfg, batch_tile_kernel<Sh, kFlRuntime, Cfg::kCfg.minb>, args, members, parity);
+    return plain ? cudaLaunchKernelEx(&cfg, batch_tile_kernel<Sh, kFlExpPlain, Cfg::kCfg.minb>, args)
+                 : cudaLaunchKernelEx(&cfg, batch_tile_kernel<Sh, kFlRuntime, Cfg::kCfg.minb>, args);
     }
   });
 }
@@ -282,10 +279,8 @@ cudaError_t launch_batch_tiles(int shape, const BatchArgs<typename Codec<S>::T, 
   template lbm::TileInfo lbm::tile_info<Q, S>(int); \
   template int lbm::step_ctas_per_sm<Q, S>();                                            \
   template cudaError_t lbm::launch_batch<Q, S>(                                          \
-      const lbm::BatchArgs<lbm::Codec<S>::T, S>&,                                         \
-      const lbm::BatchMember<lbm::Codec<S>::T, S>*, int, int, bool, bool, cudaStream_t);    \
+      const lbm::BatchArgs<Q, lbm::Codec<S>::T, S>&, int, bool, bool, cudaStream_t);          \
   template cudaError_t lbm::launch_batch_tiles<Q, S>(                                    \
-      int, const lbm::BatchArgs<lbm::Codec<S>::T, S>&,                                     \
-      const lbm::BatchMember<lbm::Codec<S>::T, S>*, int, int, bool, cudaStream_t);         \
+      int, const lbm::BatchArgs<Q, lbm::Codec<S>::T, S>&, int, bool, cudaStream_t);           \
   template cudaError_t lbm::prepare_batch_tiles<Q, S>(int);                              \
   template int lbm::batch_ctas_per_sm<Q, S>();

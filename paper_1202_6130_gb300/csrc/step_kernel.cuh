@@ -186,7 +186,7 @@ __device__ __forceinline__ uint64_t step_smem_init(const StepSmem<Q, S, W, NS>& 
 // arithmetic is the same in either direction.  Returns false if a stage never
 // arrived (the status word then has kStatusTimeout).
 template <int Q, typename S, int W, int NS, int FL, typename Args>
-__device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensorMap* flg,
+__device__ __forceinline__ bool march_segment(const CUtensorMap* src, const CUtensorMap* flg,
                                               const Args& a, int x0, int y0, int Lr, bool rev,
                                               const StepSmem<Q, S, W, NS>& sm, uint32_t& g,
                                               uint64_t policy) {
@@ -238,13 +238,13 @@ __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensor
       // the segment below a few microseconds later and should hit in L2.
       constexpr int off = Sh::kTab.box_off[j], map = Sh::kTab.box_map[j];
       constexpr int plane = Sh::kTab.box_plane[j];
-      tma_load_3d(st + off, &src->m[map], &bars[s], x0, ynode - cy + GY, plane);
+      tma_load_3d(st + off, &src[map], &bars[s], x0, ynode - cy + GY, plane);
     });
     if (wall_on) tma_load_2d(st + Sh::POP_BYTES, flg, &bars[s], (x0 >> 5) & ~3, ynode);
   };
   int issued = 0;
   if (tid == kIss) {
-    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src->m[decltype(kc)::value]); });
+    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src[decltype(kc)::value]); });
     if (wall_on) prefetch_tensormap(flg);
     const int n0 = min(NS, K);
 #pragma unroll 1
@@ -380,7 +380,7 @@ __device__ __forceinline__ bool march_segment(const PopMaps* src, const CUtensor
 // does.  Wall terms, ghost images, the halo psi and a pair that straddles the
 // lattice's right edge fall back to per-node code.
 template <int Q, typename S, int W, int NS, int FL, typename Args>
-__device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUtensorMap* flg,
+__device__ __forceinline__ bool march_segment_v2(const CUtensorMap* src, const CUtensorMap* flg,
                                                  const Args& a, int x0, int y0, int Lr, bool rev,
                                                  const StepSmem<Q, S, W, NS>& sm, uint32_t& g) {
   using Sh = StepShape<Q, S, W, NS>;
@@ -432,13 +432,13 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
       constexpr int cy = Sh::kTab.box_cy[j];
       constexpr int off = Sh::kTab.box_off[j], map = Sh::kTab.box_map[j];
       constexpr int plane = Sh::kTab.box_plane[j];
-      tma_load_3d(st + off, &src->m[map], &bars[s], x0, ynode - cy + GY, plane);
+      tma_load_3d(st + off, &src[map], &bars[s], x0, ynode - cy + GY, plane);
     });
     if (wall_on) tma_load_2d(st + Sh::POP_BYTES, flg, &bars[s], (x0 >> 5) & ~3, ynode);
   };
   int issued = 0;
   if (tid == kIss) {
-    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src->m[decltype(kc)::value]); });
+    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src[decltype(kc)::value]); });
     if (wall_on) prefetch_tensormap(flg);
     const int n0 = min(NS, K);
 #pragma unroll 1
@@ -593,7 +593,7 @@ __device__ __forceinline__ bool march_segment_v2(const PopMaps* src, const CUten
 // Marches one segment with the variant the shape selects (one or two nodes
 // per thread).
 template <int Q, typename S, int W, int NS, int FL, typename Args>
-__device__ __forceinline__ bool march_any(const PopMaps* src, const CUtensorMap* flg,
+__device__ __forceinline__ bool march_any(const CUtensorMap* src, const CUtensorMap* flg,
                                           const Args& a, int x0, int y0, int Lr, bool rev,
                                           const StepSmem<Q, S, W, NS>& sm, uint32_t& g,
                                           uint64_t policy) {
@@ -626,40 +626,42 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
   // Every CTA reads the counter in march_any before this launch ends; the
   // word written here is read only by the next step.
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) advance_key<kModeStep>(a);
-  march_any<Q, S, W, NS, FL>(&src, &flg, a, blockIdx.x * W, y0, min(a.tile_rows, a.ny - y0),
+  march_any<Q, S, W, NS, FL>(src.m, &flg, a, blockIdx.x * W, y0, min(a.tile_rows, a.ny - y0),
                                (blockIdx.y & 1u) != 0u, sm, g, policy);
   griddep_launch_dependents();
 }
 
-// A lattice of a batch: TMA maps of its two population buffers for the batch's
-// kernel and of its wall flags, and the flag words themselves (in device memory;
-// map[d] reads buffer d).
-template <typename T, typename S> struct BatchMember {
-  PopMaps map[2];
-  CUtensorMap flags;
-  const uint32_t* flag_words;
-  int32_t flag_pitch;
-};
-
-// Step arguments of up to kChunk members of a batch for either direction
-// (a[m][d] reads buffer d and writes buffer 1 - d), the buffer holding each
-// member's state at parity 0, and the chunk's tiles: member m owns tiles
-// [tile0[m], tile0[m + 1]), nseg[m] segments of nstrip[m] strips numbered
-// segment by segment (tile0[m] = the chunk's tile count past its last member).
-// Passed as a kernel parameter, so the kernel reads them from constant memory
-// with the CTA-uniform member index that it derives from its block index.
-// kChunk: 64 members with FP32 arithmetic, 32 with FP64 (the larger FP64
-// arguments), so that the block stays below the 32,764-byte parameter limit.
-template <typename T> constexpr int batch_chunk() { return sizeof(T) == 8 ? 32 : 64; }
-template <typename T, typename S> struct BatchArgs {
-  static constexpr int kChunk = batch_chunk<T>();
-  StepArgs<T, S> a[kChunk][2];
-  int32_t cur[kChunk];
+// One step of up to kChunk members of a batch: member m's TMA maps of the buffer the
+// step reads and of its wall flags (for the march) or the flag words themselves
+// (for tiles), its arguments, and its tiles [tile0[m], tile0[m + 1]): nseg[m]
+// segments of nstrip[m] strips numbered segment by segment (tile0[m] = the
+// chunk's tile count past its last member).  Passed as a kernel parameter, so
+// the kernel reads the arguments from constant memory with the CTA-uniform
+// member index that it derives from its block index, and the maps are those of
+// this launch: maps in device memory that the host rewrites between launches
+// would need a tensormap proxy fence in every CTA before their use (GB300, us
+// per step, fence / here: twelve 650x150 D2Q21 FP32 lattices 62 / 53, 48 uneven
+// D2Q9 FP32 lattices 63 / 49, 256 of them 297 / 283, FP16S 212 / 203).
+// kChunk: 64 D2Q9 members, 40 with D2Q21's three maps, 32 with FP64's larger
+// arguments.  The block stays below 31 KB: with 32,640 bytes (the documented limit
+// is 32,764) entries past about 31,900 read as zero in several kernels (nvcc
+// 13.0.88), where they pass 32 KB of the bank that holds the parameters.
+template <int Q, typename T> constexpr int batch_chunk() {
+  return sizeof(T) == 8 ? 32 : (Q == 9 ? 64 : 40);
+}
+template <int Q, typename T, typename S> struct BatchArgs {
+  static constexpr int kChunk = batch_chunk<Q, T>();
+  CUtensorMap map[kChunk][kMapsOf<Q>];
+  CUtensorMap flags[kChunk];
+  StepCore<T, S> a[kChunk];
+  const uint32_t* flag_words[kChunk];
   int32_t tile0[kChunk + 1];
   int32_t nstrip[kChunk];
   int32_t nseg[kChunk];
 };
-static_assert(sizeof(BatchArgs<float, float>) <= 32764 && sizeof(BatchArgs<double, double>) <= 32764,
+constexpr size_t kBatchArgsLimit = 31 * 1024;
+static_assert(sizeof(BatchArgs<9, float, float>) <= kBatchArgsLimit && sizeof(BatchArgs<21, float, float>) <= kBatchArgsLimit &&
+                  sizeof(BatchArgs<9, double, double>) <= kBatchArgsLimit && sizeof(BatchArgs<21, double, double>) <= kBatchArgsLimit,
               "batch arguments fit the kernel parameter space");
 
 // The member that tile t of a chunk belongs to (uniform across the CTA: t comes
@@ -675,14 +677,11 @@ template <typename Batch> __device__ __forceinline__ int batch_member(const Batc
 // t / nstrip (rows balanced over the member's height, odd segments marched
 // upwards as in step_kernel) and strip t % nstrip of its member.  With
 // PERSIST, CTA b marches tiles b, b + gridDim.x, ...; otherwise CTA b marches
-// tile b.  `parity` flips the read/write buffers on alternate steps.  FL as
-// for step_kernel (kFlExpPlain when every member of the chunk has those
+// tile b.  FL as for step_kernel (kFlExpPlain when every member of the chunk has those
 // settings).
 template <int Q, typename S, int W, int NS, int MINB, bool PERSIST, int FL>
 __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
-    batch_step_kernel(const __grid_constant__ BatchArgs<typename Codec<S>::T, S> P,
-                      const BatchMember<typename Codec<S>::T, S>* __restrict__ members,
-                      int32_t parity) {
+    batch_step_kernel(const __grid_constant__ BatchArgs<Q, typename Codec<S>::T, S> P) {
   extern __shared__ unsigned char smem_raw[];
   const auto sm = StepSmem<Q, S, W, NS>::carve(smem_raw);
   const uint64_t policy = step_smem_init(sm);
@@ -694,14 +693,12 @@ __global__ void __launch_bounds__(StepShape<Q, S, W, NS>::NT, MINB)
     const int local = t - P.tile0[m];
     const int seg = local / P.nstrip[m];
     const int x0 = (local - seg * P.nstrip[m]) * W;
-    const int dir = (P.cur[m] ^ parity) & 1;
-    const auto& a = P.a[m][dir];
+    const auto& a = P.a[m];
     const int y0 = (int)((int64_t)a.ny * seg / P.nseg[m]);
     const int y1 = (int)((int64_t)a.ny * (seg + 1) / P.nseg[m]);
     if (threadIdx.x == 0 && local == 0) advance_key<kModeStep>(a);
-    const auto* mb = &members[m];
-    return march_any<Q, S, W, NS, FL>(&mb->map[dir], &mb->flags, a, x0, y0, y1 - y0,
-                                                (seg & 1) != 0, sm, g, policy);
+    return march_any<Q, S, W, NS, FL>(P.map[m], &P.flags[m], a, x0, y0, y1 - y0, (seg & 1) != 0, sm,
+                                      g, policy);
   };
   if constexpr (PERSIST) {
     const int nt = P.tile0[P.kChunk];

@@ -112,7 +112,7 @@ template <int Q_, typename S_, int TW_, int TH_, int NT_, int TS_, bool IN_> str
   static constexpr int NMAP = kTab.nmap;
   static constexpr int SMEM = 128 /*alignment slack*/ + kTab.bytes + PW * BH * (int)sizeof(T) + 16;
   static_assert(TW % 16 == 0 && NT % 32 == 0, "tile shape");
-  static_assert(BW <= 256 && BH <= 256 && NMAP <= kMaxMaps, "tensor-map boxes");
+  static_assert(BW <= 256 && BH <= 256 && NMAP == kMapsOf<Q>, "tensor-map boxes");
   static_assert(margin(0) + 2 * R <= GX && margin(0) + 2 * R <= GY, "ghost frame");
   static_assert(TS == 1 || (TS % 2 == 0 && V == 2 && R == 1), "several steps: D2Q9 node pairs");
   static_assert(kHaloItems || R == 1, "halo columns node by node: R = 1");
@@ -122,7 +122,7 @@ template <int Q_, typename S_, int TW_, int TH_, int NT_, int TS_, bool IN_> str
 // its moments (kModeMoments, TS = 1).  (xn, yn): a later CTA's tile to fetch into
 // L2 meanwhile (xn < 0: none).
 template <typename Sh, int MODE, int FL, typename Args>
-__device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* __restrict__ flags,
+__device__ __forceinline__ void tile_update(const CUtensorMap* src, const uint32_t* __restrict__ flags,
                                             int flag_pitch, const Args& a, int x0, int y0,
                                             int xn, int yn, unsigned char* smem_raw) {
   using S = typename Sh::S;
@@ -143,7 +143,7 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
     mbar_init(bar, 1);
     *s_abort = 0;
     fence_barrier_init();
-    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src->m[decltype(kc)::value]); });
+    static_for<0, Sh::NMAP>([&](auto kc) { prefetch_tensormap(&src[decltype(kc)::value]); });
   }
   auto wrap_x = [&](int x) { return x < 0 ? x + a.nx : (x >= a.nx ? x - a.nx : x); };
   auto wrap_y = [&](int y) { return y < 0 ? y + a.ny : (y >= a.ny ? y - a.ny : y); };
@@ -201,13 +201,13 @@ __device__ __forceinline__ void tile_update(const PopMaps* src, const uint32_t* 
       constexpr int j = decltype(jc)::value;
       constexpr int cy = Sh::kTab.box_cy[j], off = Sh::kTab.box_off[j], map = Sh::kTab.box_map[j];
       constexpr int plane = Sh::kTab.box_plane[j];
-      tma_load_3d(base + off, &src->m[map], bar, x0, y0 - BR - cy + GY, plane);
+      tma_load_3d(base + off, &src[map], bar, x0, y0 - BR - cy + GY, plane);
     });
     if (xn >= 0)  // the lines of a tile some waves ahead, into L2
       static_for<0, Sh::NBOX>([&](auto jc) {
         constexpr int j = decltype(jc)::value;
         constexpr int cy = Sh::kTab.box_cy[j], map = Sh::kTab.box_map[j], plane = Sh::kTab.box_plane[j];
-        tma_prefetch_3d(&src->m[map], xn, yn - BR - cy + GY, plane);
+        tma_prefetch_3d(&src[map], xn, yn - BR - cy + GY, plane);
       });
   }
   const uint32_t key = step_key<S, MODE, FL>(a);
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(Sh::NT, MINB)
       yn = tn * Sh::TH;
     }
   }
-  tile_update<Sh, MODE, FL>(&src, flags, flag_pitch, a, blockIdx.x * Sh::TW, ty * Sh::TH, xn, yn,
+  tile_update<Sh, MODE, FL>(src.m, flags, flag_pitch, a, blockIdx.x * Sh::TW, ty * Sh::TH, xn, yn,
                             smem_raw);
   if constexpr (MODE == kModeStep)
     if (blockIdx.x == 0 && ty == 0 && threadIdx.x == 0) advance_key<MODE>(a, Sh::TS);
@@ -410,19 +410,15 @@ __global__ void __launch_bounds__(Sh::NT, MINB)
 
 // One step of up to kChunk lattices of a batch on tiles: CTA b updates tile b of
 // the chunk, numbered member by member and, within a member, row by row
-// (nstrip tiles per row).  Members and arguments as for batch_step_kernel.
+// (nstrip tiles per row).  Arguments as for batch_step_kernel.
 template <typename Sh, int FL, int MINB>
 __global__ void __launch_bounds__(Sh::NT, MINB)
-    batch_tile_kernel(const __grid_constant__ BatchArgs<typename Sh::T, typename Sh::S> P,
-                      const BatchMember<typename Sh::T, typename Sh::S>* __restrict__ members,
-                      int32_t parity) {
+    batch_tile_kernel(const __grid_constant__ BatchArgs<Sh::Q, typename Sh::T, typename Sh::S> P) {
   extern __shared__ unsigned char smem_raw[];
   const int m = batch_member(P, (int)blockIdx.x);
   const int local = (int)blockIdx.x - P.tile0[m], ty = local / P.nstrip[m];
-  const int dir = (P.cur[m] ^ parity) & 1;
-  const auto& a = P.a[m][dir];
-  const auto* mb = &members[m];
-  tile_update<Sh, kModeStep, FL>(&mb->map[dir], mb->flag_words, mb->flag_pitch, a,
+  const auto& a = P.a[m];
+  tile_update<Sh, kModeStep, FL>(P.map[m], P.flag_words[m], flag_words_per_row(a.nx), a,
                                  (local - ty * P.nstrip[m]) * Sh::TW, ty * Sh::TH, -1, 0, smem_raw);
   if (threadIdx.x == 0 && local == 0) advance_key<kModeStep>(a, Sh::TS);
 }

@@ -247,3 +247,49 @@ def test_batch_memory_comes_from_the_pool_of_the_batch_stream(pkg):
     assert p != freed
     b.allocator._free_cb(p, None)
     b.close()
+
+
+@pytest.mark.parametrize("storage,lattice", [("fp64", 9), ("fp32", 9), ("fp16s", 9), ("fp32", 21),
+                                             ("bf16s", 21)])
+def test_descriptors_rewritten_in_place_between_launches(pkg, storage, lattice):
+    """Each change of the tiling writes the members' tensor maps anew at the
+    addresses they had, with boxes of one row for a march and of a tile's height
+    for tiles, and a member that joins or leaves moves the maps of those after
+    it: every kernel reads the maps of its own launch."""
+    ws = [W.droplet_on_wall(nx=40 + 24 * k, ny=20 + 6 * k, R=6.0, seed=700 + k, noise_amp=1e-5,
+                            lattice=lattice) for k in range(5)]
+    want = [_alone(pkg, w, storage, 60) for w in ws]
+    sims = [pkg.Simulation.from_workload(w, storage=storage) for w in ws]
+    b = pkg.Batch()
+    for s in sims:
+        b.add(s)
+    for k in range(10):
+        for tiling in ((0, 0), (16, 0), (5, 7)):
+            b.set_tiling(*tiling)
+            b.step(2)
+        b.remove(sims[k % 5])
+        b.add(sims[k % 5])
+    for s, f in zip(sims, want):
+        np.testing.assert_array_equal(s.populations(), f)
+    b.close()
+
+
+@pytest.mark.parametrize("storage,lattice,n", [("fp32", 21, 41), ("bf16s", 21, 41), ("fp64", 21, 33),
+                                               ("fp64", 9, 33), ("fp32", 9, 64)])
+def test_full_chunks_equal_members_alone_bitwise(pkg, storage, lattice, n):
+    """Every entry of a launch's argument block: chunks of 40 D2Q21 members, of 32
+    with FP64 storage and of 64 otherwise, full and (but for the last case) one
+    more, on tiles, on a march and on persistent CTAs."""
+    ws = [W.droplet_on_wall(nx=16 + 2 * (k % 9), ny=14 + k % 7, R=4.0, seed=900 + k, noise_amp=1e-5,
+                            lattice=lattice, tau=0.7 + 0.01 * k) for k in range(n)]
+    sims = [pkg.Simulation.from_workload(w, storage=storage) for w in ws]
+    b = pkg.Batch()
+    for s in sims:
+        b.add(s)
+    assert b.launches_per_step() == (1 if n == 64 else 2)
+    for tiling in ((0, 0), (5, 0), (5, 40)):
+        b.set_tiling(*tiling)
+        b.step(3)
+    for s, w in zip(sims, ws):
+        np.testing.assert_array_equal(s.populations(), _alone(pkg, w, storage, 9))
+    b.close()
