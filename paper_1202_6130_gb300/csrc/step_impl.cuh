@@ -3,10 +3,29 @@
 #pragma once
 
 #include <algorithm>
+#include <mutex>
 
 #include "launch.cuh"
 
 namespace lbm {
+
+// A value computed once per device: kernel attributes and residency belong to the
+// device that was current when they were set or asked for, and a process may
+// hold lattices on several.
+template <typename T> class PerDevice {
+ public:
+  template <typename F> T get(F&& compute) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kDevices) return compute();
+    std::call_once(once_[dev], [&] { value_[dev] = compute(); });
+    return value_[dev];
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::once_flag once_[kDevices];
+  T value_[kDevices] = {};
+};
 
 // The common settings (exponential psi, no projection, stochastic rounding of
 // 16-bit storage) run kernels with them fixed at compile time.
@@ -18,10 +37,11 @@ template <int Q, typename S, int FL>
 static cudaError_t prepare_kernel() {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
-  static cudaError_t once = cudaFuncSetAttribute(
-      step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, FL>,
-      cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
-  return once;
+  static PerDevice<cudaError_t> once;
+  return once.get([] {
+    return cudaFuncSetAttribute(step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, FL>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
+  });
 }
 
 // The fused step as a programmatic dependent launch: the step may begin
@@ -60,35 +80,36 @@ cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
 template <int Q, typename S, int K, int MODE, int FL>
 static cudaError_t prepare_tile() {
   using Cfg = TileConfig<Q, S, K>;
-  static cudaError_t once = cudaFuncSetAttribute(tile_kernel<typename Cfg::Sh, MODE, FL, Cfg::kCfg.minb>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 Cfg::Sh::SMEM);
-  return once;
+  static PerDevice<cudaError_t> once;
+  return once.get([] {
+    return cudaFuncSetAttribute(tile_kernel<typename Cfg::Sh, MODE, FL, Cfg::kCfg.minb>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::Sh::SMEM);
+  });
 }
 
 static int sm_count() {
-  static int sms = [] {
+  static PerDevice<int> sms;
+  return sms.get([] {
     int dev = 0, n = 0;
     return cudaGetDevice(&dev) == cudaSuccess &&
                    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
                ? n : 0;
-  }();
-  return sms;
+  });
 }
 
 // CTAs of the K-th shape that the GPU holds at once (0 if the kernel cannot run).
 template <int Q, typename S, int K> static int tile_slots() {
   using Cfg = TileConfig<Q, S, K>;
   using Sh = typename Cfg::Sh;
-  static int slots = [] {
+  static PerDevice<int> slots;
+  return slots.get([] {
     int n = 0;
     if (prepare_tile<Q, S, K, kModeStep, kFlExpPlain>() != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &n, tile_kernel<Sh, kModeStep, kFlExpPlain, Cfg::kCfg.minb>, Sh::NT, Sh::SMEM) != cudaSuccess)
       return 0;
     return n * sm_count();
-  }();
-  return slots;
+  });
 }
 
 template <int Q, typename S, int K, int MODE, int FL>
@@ -168,15 +189,15 @@ template <int Q, typename S, int FL>
 static cudaError_t prepare_batch_kernel() {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
-  static cudaError_t once = [] {
+  static PerDevice<cudaError_t> once;
+  return once.get([] {
     cudaError_t e = cudaFuncSetAttribute(
         batch_step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::template batch_minb_tile<FL>(), false, FL>,
         cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(batch_step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::BATCH_MINB, true, FL>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
-  }();
-  return once;
+  });
 }
 
 template <int Q, typename S, int FL>
@@ -228,10 +249,11 @@ template <int Q, typename S> int batch_ctas_per_sm() {
 
 template <int Q, typename S, int K, int FL> static cudaError_t prepare_batch_tile_k() {
   using Cfg = TileConfig<Q, S, K>;
-  static cudaError_t once = cudaFuncSetAttribute(batch_tile_kernel<typename Cfg::Sh, FL, Cfg::kCfg.minb>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 Cfg::Sh::SMEM);
-  return once;
+  static PerDevice<cudaError_t> once;
+  return once.get([] {
+    return cudaFuncSetAttribute(batch_tile_kernel<typename Cfg::Sh, FL, Cfg::kCfg.minb>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::Sh::SMEM);
+  });
 }
 
 template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape) {
