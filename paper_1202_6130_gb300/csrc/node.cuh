@@ -371,15 +371,19 @@ __device__ __forceinline__ double f64_from_f32(float v) {
 // the remainder before it, the remainders being exact by a fused multiply-add
 // (a long division by words).  Their FP64 sum is the only FP64 work: two
 // additions instead of a division's dozen (the read-out of 4096x2048: FP32 367 ->
-// 99 us, BF16S 535 -> 90).  At most one unit in the last place
-// from the FP64 division (20 million random operands); operands outside the
-// range where no term can leave FP32's normal range divide in FP64.
+// 99 us, BF16S 535 -> 90).  At most one unit in the last place from the FP64
+// division (100 million random operands with rho from 2^-40 to 2^40).  The terms
+// shrink by about 2^-24 each, and a subnormal one (below 2^-126) is dropped:
+// with |h| >= 2^-66 rho the two terms that can be subnormal lose at most 2^-125
+// together, 1/128 of a unit.  F / 2 is exact or off by at most 2^-150, and where
+// the sum vanishes F has to be zero as well.  Other operands divide in FP64.
 __device__ __forceinline__ double half_force_velocity(float j, float F, float rho, float rc) {
   const float hf = __fmul_rn(0.5f, F);
   const float h = __fadd_rn(j, hf), hb = __fsub_rn(h, j);
   const float l = __fadd_rn(__fsub_rn(j, __fsub_rn(h, hb)), __fsub_rn(hf, hb));
   const float ah = fabsf(h);
-  if (!(rho >= 0x1p-40f && rho <= 0x1p40f && ah <= 0x1p60f && (ah >= 0x1p-70f || ah == 0.0f)))
+  if (!(rho >= 0x1p-40f && rho <= 0x1p40f && ah <= 0x1p60f &&
+        ((ah >= 0x1p-70f && ah >= rho * 0x1p-66f) || (ah == 0.0f && F == 0.0f))))
     return ((double)j + 0.5 * (double)F) / (double)rho;
   float q0 = __fmul_rn(h, rc);
   q0 = __fmaf_rn(__fmaf_rn(-q0, rho, h), rc, q0);

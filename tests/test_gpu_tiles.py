@@ -148,3 +148,29 @@ def test_fp32_velocity_quotient_is_within_an_ulp_of_fp64(pkg):
         want = j.astype(np.float64) / r.astype(np.float64)
         assert (np.abs(u - want) <= 2.0 ** -52 * np.abs(want)).all()
     sim.close()
+
+
+def test_fp32_velocity_quotient_at_any_density(pkg):
+    """The same for densities from 2^-44 to 2^44 and momenta down to FP32's
+    subnormal numbers (quotients whose words leave FP32's normal range are
+    divided in FP64), and for a momentum of zero under a subnormal force."""
+    ny, nx = 128, 128
+    rng = np.random.default_rng(11)
+    f = np.zeros((9, ny, nx), np.float32)
+    f[0] = np.ldexp(rng.uniform(1.0, 2.0, (ny, nx)), rng.integers(-44, 44, (ny, nx)))
+    for i, j in ((1, 3), (2, 4)):  # j_x and j_y to three words: f1 - f3 is rounded once
+        f[i] = np.ldexp(rng.uniform(-2.0, 2.0, (ny, nx)), rng.integers(-148, -44, (ny, nx)))
+        f[j] = f[i] * rng.uniform(0.0, 1.0, (ny, nx)).astype(np.float32)
+    f[1:5, ::8] = 0.0
+    for body in (0.0, 2.0 ** -149):
+        sim = pkg.Simulation(nx, ny, storage="fp32", G=0.0, body_force=(body, body))
+        sim.set_populations(f.astype(np.float64))
+        rho, ux, uy = sim.moments()
+        r = f[0].copy()
+        for i in range(1, 9):
+            r = r + f[i]
+        np.testing.assert_array_equal(rho, r.astype(np.float64))
+        for u, j in ((ux, f[1] - f[3]), (uy, f[2] - f[4])):
+            want = (j.astype(np.float64) + 0.5 * body) / r.astype(np.float64)
+            assert (np.abs(u - want) <= 2.0 ** -52 * np.abs(want)).all()
+        sim.close()
