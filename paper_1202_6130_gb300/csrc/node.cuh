@@ -227,10 +227,13 @@ template <> __device__ __forceinline__ float t_sqrt<float>(float v) { return sqr
 // (with the fused collision and neighbour sums, 2048x1024 D2Q9 637 -> 516 us
 // per step, 128x64 9.9 -> 8.4).
 // FP32 multiplies by y.
+// Where b is zero or infinite, or a is not finite, the remainder is not a number
+// and q = a y already is what the division gives (tested by its exponent, on
+// the integer pipe).
 template <typename T> __device__ __forceinline__ T div_rho(T a, T b, T y);
 template <> __device__ __forceinline__ double div_rho<double>(double a, double b, double y) {
-  const double q = a * y;
-  return fma(fma(-q, b, a), y, q);
+  const double q = a * y, r = fma(-q, b, a);
+  return (__double2hiint(r) & 0x7ff00000) == 0x7ff00000 ? q : fma(r, y, q);
 }
 template <> __device__ __forceinline__ float div_rho<float>(float a, float, float y) {
   return a * y;

@@ -174,3 +174,25 @@ def test_fp32_velocity_quotient_at_any_density(pkg):
             want = (j.astype(np.float64) + 0.5 * body) / r.astype(np.float64)
             assert (np.abs(u - want) <= 2.0 ** -52 * np.abs(want)).all()
         sim.close()
+
+
+def test_fp64_velocity_where_the_density_is_zero_or_infinite(pkg):
+    """u = j / rho as the FP64 division gives it: infinite or not a number at
+    rho = 0, zero at an infinite rho, and ordinary elsewhere."""
+    ny, nx = 6, 16
+    f = np.full((9, ny, nx), 0.1)
+    f[1] = 0.25                                    # j_x = 0.15
+    f[:, 2, 3], f[1, 2, 3], f[0, 2, 3] = 0.0, 0.25, -0.25      # rho = 0, j = (0.25, 0)
+    f[:, 4, 9] = 0.0                                           # rho = 0, j = 0
+    f[0, 1, 5] = np.inf                                        # rho infinite, j finite
+    sim = pkg.Simulation(nx, ny, storage="fp64", G=0.0)
+    sim.set_populations(f)
+    rho, ux, uy = (a.cpu().numpy() for a in sim.moments_device())
+    sim.close()
+    r = f.sum(0)
+    assert rho[2, 3] == 0.0 and rho[4, 9] == 0.0 and rho[1, 5] == np.inf
+    assert ux[2, 3] == np.inf and np.isnan(uy[2, 3])
+    assert np.isnan(ux[4, 9]) and np.isnan(uy[4, 9])
+    assert ux[1, 5] == 0.0 and uy[1, 5] == 0.0
+    ok = np.isfinite(r) & (r != 0.0)
+    np.testing.assert_allclose(ux[ok], 0.15 / r[ok], rtol=1e-13)
