@@ -293,19 +293,21 @@ int lbm_batch_size(const lbm_batch* b, int32_t* n);
  * an empty batch). */
 int lbm_batch_launches_per_step(const lbm_batch* b, int32_t* n);
 /* Tiling: with both 0 (the default) the engine picks two-dimensional tiles, one
- * CTA per tile, or row marches for all members by their sizes.  tile_rows > 0 asks for row
- * marches over segments of that many rows; ctas > 0 for that many persistent
- * CTAs dealing the segments round-robin (tile_rows 0: each member's own
- * choice). */
+ * CTA per tile, or row marches for all members by their sizes.  tile_rows > 0
+ * asks for CTAs of that many rows: the default's tiles where they have that
+ * height, else row marches over segments of that many rows; ctas > 0 for that
+ * many persistent CTAs dealing the march's segments round-robin (tile_rows 0:
+ * each member's own choice). */
 int lbm_batch_set_tiling(lbm_batch* b, int32_t tile_rows, int32_t ctas);
 /* Advances every member by nsteps time steps; enqueued on the batch stream. */
 int lbm_batch_step(lbm_batch* b, int64_t nsteps);
-/* Times each candidate tiling (the default tiles; row marches of 4..64 rows x
- * {one CTA per segment, one persistent wave}; 14 trials) for steps_per_trial
+/* Times each candidate tiling (4..64 rows per CTA x {one CTA per tile or segment,
+ * one persistent wave}; 14 trials) for steps_per_trial
  * steps (plus 18 warm-up steps) on the members
  * themselves -- so they advance by those steps -- keeps the fastest, and
- * records it for the batch's size class (see lbm_batch_use_tuned).
- * best_tile_rows is the chosen tiling's rows per CTA.  Outputs may be NULL.  Synchronises the stream. */
+ * records it for the batch's size class (see lbm_batch_use_tuned).  Passing
+ * best_tile_rows and best_ctas to lbm_batch_set_tiling selects it for the same
+ * members.  Outputs may be NULL.  Synchronises the stream. */
 int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile_rows,
                        int32_t* best_ctas, double* best_ms_per_step);
 /* The tiling lbm_batch_autotune last chose for a batch of the same lattice,

@@ -948,7 +948,7 @@ struct lbm_batch {
   std::vector<uint64_t> versions;
   std::vector<int> cur0;  // member cur at build time
   int Q = 0, storage = -1;
-  int tile_rows = 0;  // 0: the engine's choice; > 0: row march, rows per segment
+  int tile_rows = 0;  // 0: the engine's choice; > 0: rows per CTA (batch_tiling)
   int ctas = 0;       // 0: one CTA per tile; > 0: row march by that many persistent CTAs
   int shape = -1;     // tile shape of the members' kernel (-1: the row march)
   bool dirty = true;
@@ -1051,6 +1051,19 @@ template <int Q, typename S> int batch_shape(const lbm_batch* b, int* rows) {
   return shape;
 }
 
+// The tiling asked for: the tile shape and *rows as for batch_shape.  tile_rows > 0
+// with one CTA per tile is the default's tile shape where that has this height
+// (so that the pair lbm_batch_autotune reports selects what it timed), and a march
+// over segments of that many rows otherwise; persistent CTAs always march.
+template <int Q, typename S> int batch_tiling(const lbm_batch* b, int* rows) {
+  *rows = b->tile_rows;
+  if (b->ctas > 0) return -1;
+  int default_rows = 0;
+  const int shape = batch_shape<Q, S>(b, &default_rows);
+  if (b->tile_rows == 0) *rows = default_rows;
+  return b->tile_rows == 0 || (shape >= 0 && tile_list<Q, S>().t[shape].th == b->tile_rows) ? shape : -1;
+}
+
 template <int Q, typename S> int batch_build(lbm_batch* b) {
   using T = typename Codec<S>::T;
   using A = BatchArgs<Q, T, S>;
@@ -1058,8 +1071,8 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
   const int n = (int)b->members.size();
   constexpr int kChunk = A::kChunk;
   const int nchunk = (n + kChunk - 1) / kChunk;
-  int rows = b->tile_rows;
-  b->shape = b->tile_rows == 0 && b->ctas == 0 ? batch_shape<Q, S>(b, &rows) : -1;
+  int rows = 0;
+  b->shape = batch_tiling<Q, S>(b, &rows);
   b->versions.assign(n, 0);
   b->cur0.assign(n, 0);
   for (int i = 0; i < n; ++i) {
@@ -1426,20 +1439,17 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
   BCK(b, cudaGetDevice(&dev));
   BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int cps = dispatch(b->Q, b->storage, [&]<int Q, typename S>() { return batch_ctas_per_sm<Q, S>(); });
-  // Row-march candidates, and (0, 0): the tiles that batch_build picks.
-  const int rows_c[] = {0, 4, 8, 12, 16, 24, 32, 64};
+  // Rows per CTA: the default's tiles at their height, marches at the others.
+  const int rows_c[] = {4, 8, 12, 16, 24, 32, 64};
   const int ctas_c[] = {0, std::max(1, cps) * sms};
   cudaEvent_t e0, e1;
   BCK(b, cudaEventCreate(&e0));
   BCK(b, cudaEventCreate(&e1));
   double best = 1e300;
   int bt = b->tile_rows, bc = b->ctas;
+  bool tiles = false;  // the fastest so far ran tiles
   for (int tr : rows_c) {
     for (int ct : ctas_c) {
-      // 14 trials in all, as many as before the default was one of them (the
-      // members advance by each): the tallest persistent march, which never won,
-      // makes room.
-      if ((tr == 0 || tr == 64) && ct != 0) continue;
       b->tile_rows = tr;
       b->ctas = ct;
       b->dirty = true;
@@ -1458,6 +1468,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
         best = per;
         bt = tr;
         bc = ct;
+        tiles = b->shape >= 0;
       }
     }
     if (rc) break;
@@ -1465,22 +1476,15 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc) return rc;
-  b->tile_rows = bt;
+  // Tiles are kept as the default, whose shape follows the members that come.
+  b->tile_rows = tiles ? 0 : bt;
   b->ctas = bc;
   b->dirty = true;
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    g_tuned[tune_key(b)] = {bt, bc};
+    g_tuned[tune_key(b)] = {b->tile_rows, bc};
   }
-  if (best_tile_rows) {
-    *best_tile_rows = bt;
-    if (bt == 0)  // rows per CTA of the default tiling
-      dispatch(b->Q, b->storage, [&]<int Q, typename S>() -> int {
-        const int shape = batch_shape<Q, S>(b, best_tile_rows);
-        if (shape >= 0) *best_tile_rows = tile_list<Q, S>().t[shape].th;
-        return LBM_OK;
-      });
-  }
+  if (best_tile_rows) *best_tile_rows = bt;
   if (best_ctas) *best_ctas = bc;
   if (best_ms_per_step) *best_ms_per_step = best;
   return LBM_OK;

@@ -82,3 +82,36 @@ def test_a_second_device_of_the_process_runs_every_kernel(lib, lattice, storage)
             assert {l[1] for l in _launches(lib, first)} == {device}
     big = [l for l in _launches(lib) if l[4] > 48 * 1024]
     assert not big or {l[1] for l in big} == {0, 1}
+
+
+@pytest.mark.parametrize("lattice,storage", [(9, "fp32"), (9, "fp16s"), (9, "fp64"), (21, "fp32")])
+@pytest.mark.parametrize("fast", ["batch_tile_kernel", "Lb0ELi1EEEv", "Lb1ELi1EEEv"],
+                         ids=["tiles", "march", "persistent"])
+def test_autotune_reports_a_tiling_that_can_be_set(lib, lattice, storage, fast):
+    """Whichever kernel is the fastest -- tiles, a row march, a march by persistent
+    CTAs -- the pair that autotuning reports selects that kernel on another batch
+    of such members, and a batch that adopts the tuned tiling runs it as well."""
+    def batch():
+        b = ctypes.c_void_p()
+        assert lib.lbm_batch_create(None, None, ctypes.byref(b)) == 0
+        for nx, ny in ((130, 70), (64, 32), (257, 90)):
+            assert lib.lbm_batch_add(b, _ctx(lib, nx, ny, lattice, storage)) == 0
+        return b
+
+    def step(b):
+        assert lib.lbm_batch_step(b, 1) == 0
+        return _launches(lib, lib.fake_launches() - 1)[0]
+
+    lib.fake_set_fast(fast.encode())
+    b = batch()
+    rows, ctas, ms = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_double()
+    assert lib.lbm_batch_autotune(b, 4, ctypes.byref(rows), ctypes.byref(ctas), ctypes.byref(ms)) == 0
+    want = step(b)
+    assert fast in want[0] and ms.value == 1.0 and rows.value > 0
+    again = batch()
+    assert lib.lbm_batch_set_tiling(again, rows, ctas) == 0
+    assert step(again) == want
+    adopts = batch()
+    found = ctypes.c_int32()
+    assert lib.lbm_batch_use_tuned(adopts, ctypes.byref(found)) == 0 and found.value == 1
+    assert step(adopts) == want
