@@ -22,6 +22,8 @@ class TorchAllocator:
         import torch
         self.torch = torch
         self.device = torch.device(device)
+        if self.device.index is None:  # the caching allocator wants an index
+            self.device = torch.device(self.device.type, torch.cuda.current_device())
         self.stream = stream  # None: the current stream
         self._alloc = L.ALLOC_FN(self._alloc_cb)
         self._free = L.FREE_FN(self._free_cb)
