@@ -418,7 +418,7 @@ __device__ __forceinline__ void node_moments(const T (&f)[Q], T& rho, T& jx, T& 
 }
 
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return a * b; }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 // Total force on a node (Eqs. force_SC, force_SC_FS, wall_shift):
 //   F = F_FF + rho S + rho phi^eps (U_wall - u - F_FF / rho) + body force.
@@ -428,22 +428,21 @@ __device__ __forceinline__ void node_force(const Physics<T>& P, T rho, T ux, T u
                                            T sfx, T sfy, bool has_wall, T phie, T Sx, T Sy,
                                            T uwx, T uwy, T inv_rho, T& Fx, T& Fy) {
   const T mg = -P.G * psi_c;
-  // Rounded products in FP32: the same bits whether or not a kernel holds the
-  // wall terms (which decide what the compiler could fuse).
-  const T ffx = mul_rn(mg, sfx);
-  const T ffy = mul_rn(mg, sfy);
-  Fx = ffx;
-  Fy = ffy;
+  // Where the products are rounded is written out, as in PairState: left to the
+  // compiler, the copy of a kernel without the wall terms fused them with the
+  // body force and the others did not, and a node's bits depended on its tile.
   if (has_wall) {
+    const T ffx = mul_rn(mg, sfx), ffy = mul_rn(mg, sfy);
     const T flx = rho * Sx, fly = rho * Sy;
     const T rp = rho * phie;
     const T dfx = rp * (uwx - ux - div_rho<T>(ffx, rho, inv_rho));
     const T dfy = rp * (uwy - uy - div_rho<T>(ffy, rho, inv_rho));
-    Fx = ((ffx + flx) + dfx);
-    Fy = ((ffy + fly) + dfy);
+    Fx = ((ffx + flx) + dfx) + P.bfx;
+    Fy = ((ffy + fly) + dfy) + P.bfy;
+  } else {
+    Fx = fma(mg, sfx, P.bfx);
+    Fy = fma(mg, sfy, P.bfy);
   }
-  Fx += P.bfx;
-  Fy += P.bfy;
 }
 
 // Index of the velocity opposite to c_i (compile time).

@@ -196,3 +196,60 @@ def test_fp64_velocity_where_the_density_is_zero_or_infinite(pkg):
     assert ux[1, 5] == 0.0 and uy[1, 5] == 0.0
     ok = np.isfinite(r) & (r != 0.0)
     np.testing.assert_allclose(ux[ok], 0.15 / r[ok], rtol=1e-13)
+
+
+# A size that selects each tile shape of a (lattice, storage), with remainders in x
+# and y (odd widths where one-step D2Q9 shapes are to run), and the sizes at which
+# the two-step shapes run in practice.
+SHAPES = {
+    (9, "fp64"): {(16, 4, 1): [(49, 9)], (32, 8, 1): [(1457, 17), (2049, 259)],
+                  (32, 16, 1): [(193, 1267), (520, 500)]},
+    (21, "fp64"): {(16, 4, 1): [(49, 9)], (32, 8, 1): [(1459, 17)], (32, 16, 1): [(97, 435), (333, 203)]},
+    (21, "fp32"): {(16, 4, 1): [(49, 9)], (32, 8, 1): [(1258, 17), (651, 150)],
+                   (64, 8, 1): [(10769, 58), (1250, 500)]},
+    (21, "fp16s"): {(32, 4, 1): [(97, 9), (651, 150)], (64, 8, 1): [(418, 1510), (1250, 300)]},
+    (9, "fp32"): {(32, 4, 1): [(97, 9)], (64, 8, 1): [(6753, 21), (1537, 771)], (32, 4, 2): [(98, 9)],
+                  (32, 8, 2): [(134, 927), (402, 203)], (32, 28, 2): [(520, 1502), (1538, 771)],
+                  (64, 12, 2): [(5236, 33), (1026, 515)], (64, 22, 2): [(11064, 61), (2050, 1027)]},
+    (9, "fp16s"): {(32, 4, 1): [(97, 9)], (64, 8, 1): [(289, 1339), (1538, 771)], (32, 4, 2): [(98, 9)],
+                   (32, 8, 2): [(130, 739), (400, 201)], (32, 28, 2): [(130, 1526), (1026, 515)],
+                   (64, 12, 2): [(6910, 33)], (64, 22, 2): [(6606, 65), (12160, 41)]},
+}
+SHAPES[9, "bf16s"], SHAPES[21, "bf16s"] = SHAPES[9, "fp16s"], SHAPES[21, "fp16s"]
+SHAPE_CASES = [(q, st, shape, size) for (q, st), shapes in SHAPES.items()
+               for shape, sizes in shapes.items() for size in sizes]
+
+
+@pytest.mark.parametrize("lattice,storage,shape,size", SHAPE_CASES,
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_each_tile_shape_equals_the_row_march_bitwise(pkg, lattice, storage, shape, size):
+    """The shape that runs is the one meant (columns, rows and steps of a launch,
+    from the layout), and four steps and one more give the row march's bits."""
+    w = _case(*size, lattice=lattice)
+    sim = pkg.Simulation.from_workload(w, storage=storage)
+    lay = sim.layout()
+    bytes_per_step = 2 * lattice * {"fp64": 8, "fp32": 4}.get(storage, 2)
+    assert lay["stages"] == 1
+    assert (lay["strip_width"], lay["tile_rows"], bytes_per_step // lay["bytes_per_node"]) == shape
+    sim.step(4)
+    sim.step(1)
+    march = pkg.Simulation.from_workload(w, storage=storage, tile_rows=4)
+    assert march.layout()["stages"] > 1
+    march.step(5)
+    np.testing.assert_array_equal(sim.populations(), march.populations())
+    sim.close()
+    march.close()
+
+
+@pytest.mark.parametrize("lattice,storage,size", [(9, "fp64", (520, 500)), (21, "fp64", (333, 203)),
+                                                  (21, "fp32", (1250, 500)), (21, "bf16s", (1250, 300)),
+                                                  (9, "fp32", (1537, 771)), (9, "fp16s", (1026, 515))],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_shapes_with_inner_tiles_equal_the_row_march_with_run_time_switches(pkg, lattice, storage, size):
+    """The equation-of-state psi and the projection, on lattices with tiles that run
+    the copy of the update without edges and walls."""
+    w = _case(*size, lattice=lattice)
+    w.psi_kind, w.G = 1, -1.0
+    want = _run(pkg, w, storage, 4, (5,), project=True)[0]
+    assert np.isfinite(want).all()
+    np.testing.assert_array_equal(_run(pkg, w, storage, 0, (4, 1), project=True)[0], want)
