@@ -253,3 +253,42 @@ def test_shapes_with_inner_tiles_equal_the_row_march_with_run_time_switches(pkg,
     want = _run(pkg, w, storage, 4, (5,), project=True)[0]
     assert np.isfinite(want).all()
     np.testing.assert_array_equal(_run(pkg, w, storage, 0, (4, 1), project=True)[0], want)
+
+
+def test_full_size_two_step_tiles_match_oracle_and_the_row_march(pkg):
+    """Two steps of the 8192x4096 multi-droplet lattice in one launch, as the
+    benchmark takes them, after 20 steps: 70 sampled nodes (tile edges in x and y,
+    wall rows, the periodic seam) recomputed by the oracle from a periodic 11x11
+    window of the FP32 state (the reach of two steps is 4), within twice the
+    bound of one step (1e-5); and every population equal to two row marches."""
+    from oracle import lbm_oracle as O
+    w = W.large_multi_droplet(noise_amp=1e-6)
+    sim = pkg.Simulation.from_workload(w, storage="fp32")
+    lay = sim.layout()
+    tw, th = lay["strip_width"], lay["tile_rows"]
+    assert lay["stages"] == 1 and lay["bytes_per_node"] == 36     # two steps per launch
+    sim.step(20)
+    f0 = sim.populations()
+    sim.step(2)
+    f2 = sim.populations()
+    sim.close()
+    march = pkg.Simulation.from_workload(w, storage="fp32", tile_rows=4)
+    march.set_populations(f0)
+    march.step(2)
+    np.testing.assert_array_equal(f2, march.populations())
+    march.close()
+    p = O.Params(lattice=O.D2Q9, tau=w.tau, G=w.G, rho0=w.rho0, body_force=tuple(w.body_force))
+    r = 5
+    rng = np.random.default_rng(2)
+    ys = list(rng.integers(0, w.ny, 40)) + [0, 1, 2, w.ny - 1, w.ny - 2, th - 1, th, th + 1, 2 * th - 1,
+                                           2 * th] + [100 * th + d for d in range(-3, 7)]
+    xs = list(rng.integers(0, w.nx, 40)) + [0, w.nx - 1, 1, tw - 1, tw, tw + 1, 2 * tw - 1, w.nx - tw,
+                                           4095, 4096] + [50 * tw + d for d in range(-4, 6)]
+    for y, x in zip(ys, xs):
+        at = np.ix_(np.arange(y - r, y + r + 1) % w.ny, np.arange(x - r, x + r + 1) % w.nx)
+        wall = O.Wall(w.phi_s[at], w.psi_r[at], w.psi_a[at], w.G_R, w.G_A, w.epsilon)
+        fo = np.stack([f[at] for f in f0])
+        for _ in range(2):
+            fo = O.step(p, wall, fo)
+        err = np.max(np.abs(f2[:, y, x] - fo[:, r, r]) / np.maximum(np.abs(fo[:, r, r]), 1e-3))
+        assert err < 2e-5, (y, x, err)
