@@ -293,3 +293,29 @@ def test_full_chunks_equal_members_alone_bitwise(pkg, storage, lattice, n):
     for s, w in zip(sims, ws):
         np.testing.assert_array_equal(s.populations(), _alone(pkg, w, storage, 9))
     b.close()
+
+
+@pytest.mark.parametrize("lattice,storage,sizes", [
+    (9, "fp64", [(520, 500), (333, 203)]), (21, "fp64", [(333, 203), (97, 435)]),
+    (21, "fp32", [(1250, 500), (651, 150)]), (21, "bf16s", [(1250, 300), (651, 150)]),
+    (9, "fp32", [(1537, 771), (1026, 515)]), (9, "fp16s", [(1537, 771), (1026, 515)])],
+    ids=lambda v: str(v) if not isinstance(v, list) else "")
+@pytest.mark.parametrize("kw", [{}, dict(project=True)], ids=["plain", "project"])
+def test_large_members_equal_their_runs_alone_bitwise(pkg, lattice, storage, sizes, kw):
+    """Members large enough for the larger tile shapes, whose inner tiles run the
+    copy of the update without edges and walls."""
+    ws = []
+    for nx, ny in sizes:
+        w = W.droplet_on_wall(nx=nx, ny=ny, R=ny / 3.0, seed=nx, noise_amp=1e-4, lattice=lattice, tau=0.8)
+        w.body_force = (1e-5, -2e-6)
+        ws.append(w)
+    sims = [pkg.Simulation.from_workload(w, storage=storage, **kw) for w in ws]
+    b = pkg.Batch()
+    for s in sims:
+        b.add(s)
+    b.step(5)
+    for s, w in zip(sims, ws):
+        want = _alone(pkg, w, storage, 5, **kw)
+        assert np.isfinite(want).all()
+        np.testing.assert_array_equal(s.populations(), want)
+    b.close()
