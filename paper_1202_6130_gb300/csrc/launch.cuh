@@ -58,7 +58,10 @@ cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
 // and the microseconds of a launch, us0 + us per round of resident CTAs (FP64: per
 // tile of the SM with the most tiles), fitted to GB300 times on 128x64 to 4096x2048 lattices (within about 15%).  The shape with
 // the least time per step by this estimate runs (choose_tiles); on the lattices
-// of the fit that is the fastest one or within 6% of it.
+// of the fit that is the fastest one or within 6% of it.  (At these register
+// budgets the 64-wide D2Q9 and 16-bit D2Q21 shapes and the 32x28 one spill: 4-16
+// bytes with the common settings fixed at compile time, 32-72 with all of them
+// at run time.)
 struct TileCfg {
   int tw, th, nt, steps;
   bool in;

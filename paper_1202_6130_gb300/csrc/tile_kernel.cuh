@@ -18,12 +18,14 @@
 // Two steps per launch (TS = 2, D2Q9 node pairs): the tile's populations stay in
 // shared memory between the steps, so a pair of steps costs one launch, one load
 // latency and one trip through HBM; the price is the first step on 2 more nodes
-// on every side (8x larger tiles for the lattices that can afford them).  GB300,
-// us per step, best one-step kernel -> two steps: 128x64 FP32 3.0 -> 2.1, 400x200
-// FP32 4.3 -> 2.9, 1024x512 FP32 8.3 -> 7.6, 4096x2048 FP32 96 -> 80 (its DRAM
-// traffic halves; what bounds it then is latency between barriers at 20 warps
-// per SM, 45% of issue slots), 8192x4096 FP32 368 -> 304.  16-bit storage is
-// bound by instruction issue on large lattices and stays at one step there.
+// on every side (larger tiles for the lattices that can afford them).  GB300, us
+// per step, best one-step kernel -> two steps when they came -> with the shapes of
+// launch.cuh, wall fields ahead of the wait and boxes fetched ahead into L2:
+// 128x64 FP32 3.0 -> 2.1 -> 1.7, 400x200 FP32 4.3 -> 2.9 -> 2.4, 1024x512 FP32 8.3 ->
+// 7.6 -> 7.3, 4096x2048 FP32 96 -> 80 -> 76, 8192x4096 FP32 368 -> 304 -> 290.  The DRAM
+// traffic of the large ones halves; what bounds them then is latency between
+// barriers, at 28 warps per SM and 52% of issue slots.  16-bit storage is bound by
+// instruction issue on large lattices and stays at one step there.
 //
 // Tried and dropped: persistent CTAs that prefetch the next tile's boxes under
 // the last collision (loop-invariant values took the registers: 184-628 bytes
