@@ -28,6 +28,7 @@ using namespace lbm;
 struct lbm_ctx {
   lbm_params p{};
   int Q = 9, R = 1, GX = 0, GY = 0, esize = 4, W = 128, NS = 8;
+  int device = 0;  // current when the context was made
   int64_t pitch = 0, rows = 0, plane = 0;
   void* buf[2] = {nullptr, nullptr};
   int cur = 0;  // buffer holding the current state
@@ -208,7 +209,7 @@ template <int Q, typename S> int ready_tile_maps(lbm_ctx* c, int use) {
   if (c->shape[use] < 0 || c->tile_ready[use]) return LBM_OK;
   EncodeFn enc = get_encode();
   if (!enc) return fail(c, LBM_ECUDA, "cuTensorMapEncodeTiled entry point unavailable");
-  const TileInfo t = tile_info<Q, S>(c->shape[use]);
+  const TileInfo t = tile_info<Q, S>(c->shape[use], c->device);
   if (t.slots <= 0) return fail(c, LBM_ECUDA, "tile kernel cannot be resident (%s)", cudaGetErrorString(cudaGetLastError()));
   cuuint64_t dims[3] = {(cuuint64_t)(c->p.nx + 2 * c->GX), (cuuint64_t)c->rows, (cuuint64_t)Q};
   cuuint64_t strides[2] = {(cuuint64_t)(c->pitch * sizeof(S)), (cuuint64_t)(c->plane * sizeof(S))};
@@ -230,8 +231,8 @@ template <int Q, typename S> int ready_tile_maps(lbm_ctx* c, int use) {
 // Estimated microseconds of a launch of `tiles` tiles of shape k.  FP64 is bound by
 // the FP64 pipe of the SM with the most tiles; the others by latency, which
 // further CTAs on an SM share.
-template <int Q, typename S> double tile_cost(int k, int64_t tiles) {
-  const TileInfo t = tile_info<Q, S>(k);
+template <int Q, typename S> double tile_cost(int k, int64_t tiles, int device) {
+  const TileInfo t = tile_info<Q, S>(k, device);
   if (t.slots <= 0) return 1e30;
   constexpr TileList list = tile_list<Q, S>();
   const TileCfg& c = list.t[k];
@@ -262,7 +263,7 @@ template <int Q, typename S> void choose_tiles(lbm_ctx* c) {
     if (use == lbm_ctx::kTwo && (c->p.nx % 2 || c->p.nx < 4 || c->p.ny < 4)) continue;
     if (march && (use == lbm_ctx::kOne || sizeof(S) == 2)) continue;
     const int64_t tiles = (int64_t)((c->p.nx + t.tw - 1) / t.tw) * ((c->p.ny + t.th - 1) / t.th);
-    const double us = tile_cost<Q, S>(k, tiles) / t.steps;
+    const double us = tile_cost<Q, S>(k, tiles, c->device) / t.steps;
     if (us < best[use]) {
       best[use] = us;
       c->shape[use] = k;
@@ -310,11 +311,11 @@ template <int Q, typename S> int setup_layout(lbm_ctx* c) {
     int rc = make_tmap<Q, S>(c, b);
     if (rc) return rc;
   }
+  int sms = 0;
+  CK(c, cudaGetDevice(&c->device));
+  CK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
   choose_tiles<Q, S>(c);
-  int dev = 0, sms = 0;
-  CK(c, cudaGetDevice(&dev));
-  CK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int cps = step_ctas_per_sm<Q, S>();
+  const int cps = step_ctas_per_sm<Q, S>(c->device);
   if (cps <= 0) {
     cudaError_t e = cudaGetLastError();
     return fail(c, LBM_ECUDA, "step kernel cannot be resident (%s)", cudaGetErrorString(e));
@@ -393,7 +394,7 @@ int run_moments(lbm_ctx* c, double* o_rho, double* o_ux, double* o_uy, int momen
   if (int rc = ready_tile_maps<Q, S>(c, lbm_ctx::kRead)) return rc;
   const auto a = make_args<Q, S>(c, c->cur, nullptr, o_rho, o_ux, o_uy, momentum);
   CK(c, launch_tile<Q, S>(c->shape[lbm_ctx::kRead], c->tile_map[lbm_ctx::kRead][c->cur], c->wall_flags,
-                          c->nchunk_pad, a, c->stream, kModeMoments));
+                          c->nchunk_pad, a, c->device, c->stream, kModeMoments));
   return LBM_OK;
 }
 
@@ -403,12 +404,12 @@ template <int Q, typename S> int run_steps(lbm_ctx* c, int use) {
   const auto a = make_args<Q, S>(c, c->cur, static_cast<S*>(c->buf[c->cur ^ 1]), nullptr, nullptr, nullptr, 0);
   if (c->shape[use] >= 0) {
     CK(c, launch_tile<Q, S>(c->shape[use], c->tile_map[use][c->cur], c->wall_flags, c->nchunk_pad, a,
-                            c->stream, kModeStep));
+                            c->device, c->stream, kModeStep));
     return LBM_OK;
   }
   // Without walls the flag map is never read; the population map stands in.
   const CUtensorMap& fm = c->has_wall ? c->flag_map : c->tmap[c->cur].m[0];
-  CK(c, launch_step<Q, S>(c->tmap[c->cur], fm, a, dim3(c->grid_x, c->grid_y), c->stream));
+  CK(c, launch_step<Q, S>(c->tmap[c->cur], fm, a, dim3(c->grid_x, c->grid_y), c->device, c->stream));
   return LBM_OK;
 }
 
@@ -1028,6 +1029,7 @@ void release_chunk(lbm_batch::Chunk& ch) {
 // 10.8 M 115 / 106, 22.0 M 234 / 203; FP32 65 / 71, 105 / 100, 150 / 140, 309 / 282.
 template <int Q, typename S> int batch_shape(const lbm_batch* b, int* rows) {
   constexpr TileList list = tile_list<Q, S>();
+  const int device = b->members[0]->device;
   double best = 1e30, rounds = 0.0;
   int shape = -1;
   for (int k = 0; k < list.n; ++k) {
@@ -1036,11 +1038,11 @@ template <int Q, typename S> int batch_shape(const lbm_batch* b, int* rows) {
     int64_t tiles = 0;
     for (const lbm_ctx* c : b->members)
       tiles += (int64_t)((c->p.nx + t.tw - 1) / t.tw) * ((c->p.ny + t.th - 1) / t.th);
-    const double us = tile_cost<Q, S>(k, tiles);
+    const double us = tile_cost<Q, S>(k, tiles, device);
     if (us < best && tiles < (int64_t)1 << 30) {
       best = us;
       shape = k;
-      rounds = (double)tiles / tile_info<Q, S>(k).slots;
+      rounds = (double)tiles / tile_info<Q, S>(k, device).slots;
     }
   }
   *rows = 0;
@@ -1157,8 +1159,8 @@ template <int Q, typename S> int batch_build(lbm_batch* b) {
   }
   if (nchunk > 1 && !b->fork_ev) BCK(b, cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming));
   // The kernels' shared-memory attributes, outside any capture.
-  if (b->shape >= 0) BCK(b, prepare_batch_tiles<Q, S>(b->shape));
-  else batch_ctas_per_sm<Q, S>();
+  if (b->shape >= 0) BCK(b, prepare_batch_tiles<Q, S>(b->shape, b->members[0]->device));
+  else batch_ctas_per_sm<Q, S>(b->members[0]->device);
   BCK(b, cudaStreamSynchronize(b->stream));  // replays of the graphs dropped below are over
   b->phase = 0;
   drop_graph(b);
@@ -1177,7 +1179,7 @@ template <int Q, typename S> cudaError_t batch_launch(lbm_batch* b, int parity) 
     const cudaError_t e =
         b->shape >= 0
             ? launch_batch_tiles<Q, S>(b->shape, args, ch.nctas, ch.plain, st)
-            : launch_batch<Q, S>(args, ch.nctas, b->ctas > 0, ch.plain, st);
+            : launch_batch<Q, S>(args, ch.nctas, b->ctas > 0, ch.plain, b->members[0]->device, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1438,7 +1440,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t steps_per_trial, int32_t* best_tile
   int dev = 0, sms = 0;
   BCK(b, cudaGetDevice(&dev));
   BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int cps = dispatch(b->Q, b->storage, [&]<int Q, typename S>() { return batch_ctas_per_sm<Q, S>(); });
+  const int cps = dispatch(b->Q, b->storage, [&]<int Q, typename S>() { return batch_ctas_per_sm<Q, S>(dev); });
   // Rows per CTA: the default's tiles at their height, marches at the others.
   const int rows_c[] = {4, 8, 12, 16, 24, 32, 64};
   const int ctas_c[] = {0, std::max(1, cps) * sms};

@@ -46,10 +46,10 @@ template <int Q, typename S> struct StepConfig {
 template <int Q, typename S>
 using ConfigShape = StepShape<Q, S, StepConfig<Q, S>::W, StepConfig<Q, S>::NS>;
 
-// Launches the fused step as a row march.
+// Launches the fused step as a row march.  (device, here and below: the lattice's.)
 template <int Q, typename S>
 cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
-                        const StepArgs<typename Codec<S>::T, S>& a, dim3 grid,
+                        const StepArgs<typename Codec<S>::T, S>& a, dim3 grid, int device,
                         cudaStream_t stream);
 
 // Shapes of the tile kernel per (lattice, storage): tile width and height,
@@ -116,17 +116,18 @@ template <int Q, typename S, int K> struct TileConfig {
 // (kModeMoments; the list's `moments` shape only).
 template <int Q, typename S>
 cudaError_t launch_tile(int shape, const PopMaps& src, const uint32_t* flags, int flag_pitch,
-                        const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream, int mode);
+                        const StepArgs<typename Codec<S>::T, S>& a, int device, cudaStream_t stream,
+                        int mode);
 
 // What the host needs of a tile shape: its TMA boxes, and the tiles that one
 // round of resident CTAs takes (0 if the kernel cannot run).
 struct TileInfo {
   int bw, bh, nmap, depth[kMaxMaps], slots, sms;
 };
-template <int Q, typename S> TileInfo tile_info(int shape);
+template <int Q, typename S> TileInfo tile_info(int shape, int device);
 
 // CTAs of the step kernel that fit on one SM (occupancy query).
-template <int Q, typename S> int step_ctas_per_sm();
+template <int Q, typename S> int step_ctas_per_sm(int device);
 
 // One time step of up to BatchArgs::kChunk members of a batch: nctas CTAs, one per
 // tile of the chunk, or (persistent) each marching every nctas-th tile; and
@@ -135,15 +136,15 @@ template <int Q, typename S> int step_ctas_per_sm();
 // the kernel with those settings fixed runs.
 template <int Q, typename S>
 cudaError_t launch_batch(const BatchArgs<Q, typename Codec<S>::T, S>& args, int nctas,
-                         bool persistent, bool plain, cudaStream_t stream);
-template <int Q, typename S> int batch_ctas_per_sm();
+                         bool persistent, bool plain, int device, cudaStream_t stream);
+template <int Q, typename S> int batch_ctas_per_sm(int device);
 
 // The same on tiles of shape `shape`, one CTA per tile.
 template <int Q, typename S>
 cudaError_t launch_batch_tiles(int shape, const BatchArgs<Q, typename Codec<S>::T, S>& args,
                                int ntiles, bool plain, cudaStream_t stream);
 // Sets the shared-memory attribute of its kernels (outside any stream capture).
-template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape);
+template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape, int device);
 
 // Auxiliary kernels (aux.cu).
 template <int Q, typename S>

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "launch.cuh"
@@ -11,19 +12,29 @@ namespace lbm {
 
 // A value computed once per device: kernel attributes and residency belong to the
 // device that was current when they were set or asked for, and a process may
-// hold lattices on several.
+// hold lattices on several.  The caller names its lattice's device, which is
+// current for any launch that can succeed: asking the runtime each time cost
+// 0.1 us of a launch's 2.2 on the host.
 template <typename T> class PerDevice {
  public:
-  template <typename F> T get(F&& compute) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kDevices) return compute();
-    std::call_once(once_[dev], [&] { value_[dev] = compute(); });
-    return value_[dev];
+  template <typename F> T get(int device, F&& compute) {
+    if (device < 0 || device >= kDevices) return compute();
+    if (!ready_[device].load(std::memory_order_acquire)) {
+      int current = -1;
+      if (cudaGetDevice(&current) != cudaSuccess || current != device) return compute();
+      std::lock_guard<std::mutex> lock(mu_);
+      if (!ready_[device].load(std::memory_order_relaxed)) {
+        value_[device] = compute();
+        ready_[device].store(true, std::memory_order_release);
+      }
+    }
+    return value_[device];
   }
 
  private:
   static constexpr int kDevices = 64;
-  std::once_flag once_[kDevices];
+  std::mutex mu_;
+  std::atomic<bool> ready_[kDevices] = {};
   T value_[kDevices] = {};
 };
 
@@ -34,11 +45,11 @@ template <typename T, typename S> static bool plain_flags(const StepArgs<T, S>& 
 }
 
 template <int Q, typename S, int FL>
-static cudaError_t prepare_kernel() {
+static cudaError_t prepare_kernel(int device) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
   static PerDevice<cudaError_t> once;
-  return once.get([] {
+  return once.get(device, [] {
     return cudaFuncSetAttribute(step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, FL>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
   });
@@ -50,11 +61,11 @@ static cudaError_t prepare_kernel() {
 template <int Q, typename S, int FL>
 static cudaError_t launch_step_pdl(const PopMaps& src, const CUtensorMap& flags,
                                    const StepArgs<typename Codec<S>::T, S>& a, dim3 grid,
-                                   cudaStream_t stream) {
+                                   int device, cudaStream_t stream) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
   cudaError_t e;
-  if ((e = prepare_kernel<Q, S, FL>()) != cudaSuccess) return e;
+  if ((e = prepare_kernel<Q, S, FL>(device)) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(Sh::NT);
@@ -71,58 +82,57 @@ static cudaError_t launch_step_pdl(const PopMaps& src, const CUtensorMap& flags,
 
 template <int Q, typename S>
 cudaError_t launch_step(const PopMaps& src, const CUtensorMap& flags,
-                        const StepArgs<typename Codec<S>::T, S>& a, dim3 grid,
+                        const StepArgs<typename Codec<S>::T, S>& a, dim3 grid, int device,
                         cudaStream_t stream) {
-  return plain_flags(a) ? launch_step_pdl<Q, S, kFlExpPlain>(src, flags, a, grid, stream)
-                        : launch_step_pdl<Q, S, kFlRuntime>(src, flags, a, grid, stream);
+  return plain_flags(a) ? launch_step_pdl<Q, S, kFlExpPlain>(src, flags, a, grid, device, stream)
+                        : launch_step_pdl<Q, S, kFlRuntime>(src, flags, a, grid, device, stream);
 }
 
 template <int Q, typename S, int K, int MODE, int FL>
-static cudaError_t prepare_tile() {
+static cudaError_t prepare_tile(int device) {
   using Cfg = TileConfig<Q, S, K>;
   static PerDevice<cudaError_t> once;
-  return once.get([] {
+  return once.get(device, [] {
     return cudaFuncSetAttribute(tile_kernel<typename Cfg::Sh, MODE, FL, Cfg::kCfg.minb>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::Sh::SMEM);
   });
 }
 
-static int sm_count() {
+static int sm_count(int device) {
   static PerDevice<int> sms;
-  return sms.get([] {
-    int dev = 0, n = 0;
-    return cudaGetDevice(&dev) == cudaSuccess &&
-                   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
-               ? n : 0;
+  return sms.get(device, [=] {
+    int n = 0;
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) == cudaSuccess ? n : 0;
   });
 }
 
 // CTAs of the K-th shape that the GPU holds at once (0 if the kernel cannot run).
-template <int Q, typename S, int K> static int tile_slots() {
+template <int Q, typename S, int K> static int tile_slots(int device) {
   using Cfg = TileConfig<Q, S, K>;
   using Sh = typename Cfg::Sh;
   static PerDevice<int> slots;
-  return slots.get([] {
+  return slots.get(device, [=] {
     int n = 0;
-    if (prepare_tile<Q, S, K, kModeStep, kFlExpPlain>() != cudaSuccess ||
+    if (prepare_tile<Q, S, K, kModeStep, kFlExpPlain>(device) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &n, tile_kernel<Sh, kModeStep, kFlExpPlain, Cfg::kCfg.minb>, Sh::NT, Sh::SMEM) != cudaSuccess)
       return 0;
-    return n * sm_count();
+    return n * sm_count(device);
   });
 }
 
 template <int Q, typename S, int K, int MODE, int FL>
 static cudaError_t launch_tile_k(const PopMaps& src, const uint32_t* flags, int flag_pitch,
-                                 const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream) {
+                                 const StepArgs<typename Codec<S>::T, S>& a, int device,
+                                 cudaStream_t stream) {
   using Cfg = TileConfig<Q, S, K>;
   using Sh = typename Cfg::Sh;
-  cudaError_t e = prepare_tile<Q, S, K, MODE, FL>();
+  cudaError_t e = prepare_tile<Q, S, K, MODE, FL>(device);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   const int nty = (a.ny + Sh::TH - 1) / Sh::TH;
   cfg.gridDim = dim3((a.nx + Sh::TW - 1) / Sh::TW);
-  const int slots = Sh::IN ? tile_slots<Q, S, K>() : 0;
+  const int slots = Sh::IN ? tile_slots<Q, S, K>(device) : 0;
   const int ahead = (int64_t)cfg.gridDim.x * nty > slots ? slots / 2 : 0;
   cfg.blockDim = dim3(Sh::NT);
   cfg.dynamicSmemBytes = Sh::SMEM;
@@ -148,35 +158,36 @@ template <int Q, typename S, int K = 0, typename F> auto with_shape(int shape, F
 
 template <int Q, typename S>
 cudaError_t launch_tile(int shape, const PopMaps& src, const uint32_t* flags, int flag_pitch,
-                        const StepArgs<typename Codec<S>::T, S>& a, cudaStream_t stream, int mode) {
+                        const StepArgs<typename Codec<S>::T, S>& a, int device, cudaStream_t stream,
+                        int mode) {
   if (mode == kModeMoments)
     return launch_tile_k<Q, S, tile_list<Q, S>().moments, kModeMoments, kFlRuntime>(
-        src, flags, flag_pitch, a, stream);
+        src, flags, flag_pitch, a, device, stream);
   return with_shape<Q, S>(shape, [&]<int K>() {
     if constexpr (Q == 9 && sizeof(S) == 2)
       if (a.phys.psi_kind == 0 && !a.phys.project && !a.stochastic)
-        return launch_tile_k<Q, S, K, kModeStep, kFlExpNearest>(src, flags, flag_pitch, a, stream);
-    return plain_flags(a) ? launch_tile_k<Q, S, K, kModeStep, kFlExpPlain>(src, flags, flag_pitch, a, stream)
-                          : launch_tile_k<Q, S, K, kModeStep, kFlRuntime>(src, flags, flag_pitch, a, stream);
+        return launch_tile_k<Q, S, K, kModeStep, kFlExpNearest>(src, flags, flag_pitch, a, device, stream);
+    return plain_flags(a) ? launch_tile_k<Q, S, K, kModeStep, kFlExpPlain>(src, flags, flag_pitch, a, device, stream)
+                          : launch_tile_k<Q, S, K, kModeStep, kFlRuntime>(src, flags, flag_pitch, a, device, stream);
   });
 }
 
-template <int Q, typename S> TileInfo tile_info(int shape) {
+template <int Q, typename S> TileInfo tile_info(int shape, int device) {
   return with_shape<Q, S>(shape, [&]<int K>() {
     using Cfg = TileConfig<Q, S, K>;
     using Sh = typename Cfg::Sh;
     TileInfo t{Sh::BW, Sh::BH, Sh::NMAP, {}, 0, 0};
     for (int k = 0; k < Sh::NMAP; ++k) t.depth[k] = Sh::kTab.depth[k];
-    t.slots = tile_slots<Q, S, K>();
-    t.sms = sm_count();
+    t.slots = tile_slots<Q, S, K>(device);
+    t.sms = sm_count(device);
     return t;
   });
 }
 
-template <int Q, typename S> int step_ctas_per_sm() {
+template <int Q, typename S> int step_ctas_per_sm(int device) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
-  if (prepare_kernel<Q, S, kFlRuntime>() != cudaSuccess) return 0;
+  if (prepare_kernel<Q, S, kFlRuntime>(device) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
           &n, step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::MINB, kFlRuntime>, Sh::NT,
@@ -186,11 +197,11 @@ template <int Q, typename S> int step_ctas_per_sm() {
 }
 
 template <int Q, typename S, int FL>
-static cudaError_t prepare_batch_kernel() {
+static cudaError_t prepare_batch_kernel(int device) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
   static PerDevice<cudaError_t> once;
-  return once.get([] {
+  return once.get(device, [] {
     cudaError_t e = cudaFuncSetAttribute(
         batch_step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::template batch_minb_tile<FL>(), false, FL>,
         cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
@@ -202,10 +213,10 @@ static cudaError_t prepare_batch_kernel() {
 
 template <int Q, typename S, int FL>
 static cudaError_t launch_batch_fl(const BatchArgs<Q, typename Codec<S>::T, S>& args, int nctas,
-                                   bool persistent, cudaStream_t stream) {
+                                   bool persistent, int device, cudaStream_t stream) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
-  cudaError_t e = prepare_batch_kernel<Q, S, FL>();
+  cudaError_t e = prepare_batch_kernel<Q, S, FL>(device);
   if (e != cudaSuccess) return e;
   // A programmatic dependent launch, as for the single-lattice step.
   cudaLaunchConfig_t cfg = {};
@@ -227,18 +238,18 @@ static cudaError_t launch_batch_fl(const BatchArgs<Q, typename Codec<S>::T, S>& 
 
 template <int Q, typename S>
 cudaError_t launch_batch(const BatchArgs<Q, typename Codec<S>::T, S>& args, int nctas,
-                         bool persistent, bool plain, cudaStream_t stream) {
-  return plain ? launch_batch_fl<Q, S, kFlExpPlain>(args, nctas, persistent, stream)
-               : launch_batch_fl<Q, S, kFlRuntime>(args, nctas, persistent, stream);
+                         bool persistent, bool plain, int device, cudaStream_t stream) {
+  return plain ? launch_batch_fl<Q, S, kFlExpPlain>(args, nctas, persistent, device, stream)
+               : launch_batch_fl<Q, S, kFlRuntime>(args, nctas, persistent, device, stream);
 }
 
 // Residency per SM of the persistent batch kernel; also sets the shared-memory
 // attribute of every batch kernel variant (outside any stream capture).
-template <int Q, typename S> int batch_ctas_per_sm() {
+template <int Q, typename S> int batch_ctas_per_sm(int device) {
   using Cfg = StepConfig<Q, S>;
   using Sh = ConfigShape<Q, S>;
-  if (prepare_batch_kernel<Q, S, kFlRuntime>() != cudaSuccess) return 0;
-  if (prepare_batch_kernel<Q, S, kFlExpPlain>() != cudaSuccess) return 0;
+  if (prepare_batch_kernel<Q, S, kFlRuntime>(device) != cudaSuccess) return 0;
+  if (prepare_batch_kernel<Q, S, kFlExpPlain>(device) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
           &n, batch_step_kernel<Q, S, Cfg::W, Cfg::NS, Cfg::BATCH_MINB, true, kFlRuntime>, Sh::NT,
@@ -247,21 +258,21 @@ template <int Q, typename S> int batch_ctas_per_sm() {
   return n;
 }
 
-template <int Q, typename S, int K, int FL> static cudaError_t prepare_batch_tile_k() {
+template <int Q, typename S, int K, int FL> static cudaError_t prepare_batch_tile_k(int device) {
   using Cfg = TileConfig<Q, S, K>;
   static PerDevice<cudaError_t> once;
-  return once.get([] {
+  return once.get(device, [] {
     return cudaFuncSetAttribute(batch_tile_kernel<typename Cfg::Sh, FL, Cfg::kCfg.minb>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::Sh::SMEM);
   });
 }
 
-template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape) {
+template <int Q, typename S> cudaError_t prepare_batch_tiles(int shape, int device) {
   return with_shape<Q, S>(shape, [&]<int K>() {
     if constexpr (TileConfig<Q, S, K>::kCfg.steps != 1) return cudaErrorInvalidValue;
     else {
-    const cudaError_t e = prepare_batch_tile_k<Q, S, K, kFlExpPlain>();
-    return e != cudaSuccess ? e : prepare_batch_tile_k<Q, S, K, kFlRuntime>();
+    const cudaError_t e = prepare_batch_tile_k<Q, S, K, kFlExpPlain>(device);
+    return e != cudaSuccess ? e : prepare_batch_tile_k<Q, S, K, kFlRuntime>(device);
     }
   });
 }
@@ -296,13 +307,13 @@ cudaError_t launch_batch_tiles(int shape, const BatchArgs<Q, typename Codec<S>::
 #define LBM_INSTANTIATE_STEP(Q, S)                                                         \
   template cudaError_t lbm::launch_step<Q, S>(const PopMaps&, const CUtensorMap&,      \
                                               const lbm::StepArgs<lbm::Codec<S>::T, S>&,   \
-                                              dim3, cudaStream_t);                         \
-  template cudaError_t lbm::launch_tile<Q, S>(int, const PopMaps&, const uint32_t*, int, const lbm::StepArgs<lbm::Codec<S>::T, S>&, cudaStream_t, int); \
-  template lbm::TileInfo lbm::tile_info<Q, S>(int); \
-  template int lbm::step_ctas_per_sm<Q, S>();                                            \
+                                              dim3, int, cudaStream_t);                    \
+  template cudaError_t lbm::launch_tile<Q, S>(int, const PopMaps&, const uint32_t*, int, const lbm::StepArgs<lbm::Codec<S>::T, S>&, int, cudaStream_t, int); \
+  template lbm::TileInfo lbm::tile_info<Q, S>(int, int); \
+  template int lbm::step_ctas_per_sm<Q, S>(int);                                         \
   template cudaError_t lbm::launch_batch<Q, S>(                                          \
-      const lbm::BatchArgs<Q, lbm::Codec<S>::T, S>&, int, bool, bool, cudaStream_t);          \
+      const lbm::BatchArgs<Q, lbm::Codec<S>::T, S>&, int, bool, bool, int, cudaStream_t);     \
   template cudaError_t lbm::launch_batch_tiles<Q, S>(                                    \
       int, const lbm::BatchArgs<Q, lbm::Codec<S>::T, S>&, int, bool, cudaStream_t);           \
-  template cudaError_t lbm::prepare_batch_tiles<Q, S>(int);                              \
-  template int lbm::batch_ctas_per_sm<Q, S>();
+  template cudaError_t lbm::prepare_batch_tiles<Q, S>(int, int);                         \
+  template int lbm::batch_ctas_per_sm<Q, S>(int);
