@@ -368,33 +368,35 @@ __device__ __forceinline__ double f64_from_f32(float v) {
   return __hiloint2double((int)hi, zero ? 0 : (int)(b << 29));
 }
 
-// (j + F / 2) / rho as an FP64 quotient of FP32 numbers, rc the correctly rounded
-// 1 / rho.  The numerator is split exactly into two FP32 terms (Knuth's
-// two-sum) and the quotient into three: each is the leading FP32 quotient of
-// the remainder before it, the remainders being exact by a fused multiply-add
-// (a long division by words).  Their FP64 sum is the only FP64 work: two
-// additions instead of a division's dozen (the read-out of 4096x2048: FP32 367 ->
-// 99 us, BF16S 535 -> 90).  At most one unit in the last place from the FP64
-// division (100 million random operands with rho from 2^-40 to 2^40).  The terms
-// shrink by about 2^-24 each, and a subnormal one (below 2^-126) is dropped:
-// with |h| >= 2^-66 rho the two terms that can be subnormal lose at most 2^-125
-// together, 1/128 of a unit.  F / 2 is exact or off by at most 2^-150, and where
-// the sum vanishes F has to be zero as well.  Other operands divide in FP64.
-__device__ __forceinline__ double half_force_velocity(float j, float F, float rho, float rc) {
-  const float hf = __fmul_rn(0.5f, F);
-  const float h = __fadd_rn(j, hf), hb = __fsub_rn(h, j);
-  const float l = __fadd_rn(__fsub_rn(j, __fsub_rn(h, hb)), __fsub_rn(hf, hb));
+// (j + F / 2) / rho as an FP64 quotient of FP32 numbers, formed as (2 j + F) / (2 rho):
+// r2 = 2 rho, rc2 the correctly rounded 1 / r2.  The numerator is split exactly
+// into two FP32 terms (Knuth's two-sum) and the quotient into three: each is the
+// leading FP32 quotient of the remainder before it, the remainders being exact by
+// a fused multiply-add (a long division by words).  Their FP64 sum is the only
+// FP64 work: two additions instead of a division's dozen (the read-out of
+// 4096x2048: FP32 367 -> 99 us, BF16S 535 -> 90).  At most one unit in the last
+// place from the FP64 division (100 million random operands with rho from 2^-40
+// to 2^40).  The terms shrink by about 2^-24 each, and a subnormal one (below
+// 2^-126) is dropped: with |h| >= 2^-72 r2 that loses at most 2^-126, a quarter of
+// a unit.  Other operands divide in FP64.  (The bound is no narrower than that,
+// and one comparison: at rest under a wall that does not vary along x, h is the
+// rounding residue of S_x, about 2^-63; with a bound of 2^-66 a read-out of 128x64
+// FP16S took 3.35 us instead of 2.66, with two comparisons 2.71.)
+__device__ __forceinline__ double half_force_velocity(float j, float F, float rho, float r2, float rc2) {
+  const float j2 = __fadd_rn(j, j);
+  const float h = __fadd_rn(j2, F), hb = __fsub_rn(h, j2);
+  const float l = __fadd_rn(__fsub_rn(j2, __fsub_rn(h, hb)), __fsub_rn(F, hb));
   const float ah = fabsf(h);
-  if (!(rho >= 0x1p-40f && rho <= 0x1p40f && ah <= 0x1p60f &&
-        ((ah >= 0x1p-70f && ah >= rho * 0x1p-66f) || (ah == 0.0f && F == 0.0f))))
+  if (!(r2 >= 0x1p-39f && r2 <= 0x1p41f && ah <= 0x1p61f &&
+        (ah >= fmaxf(0x1p-69f, r2 * 0x1p-72f) || ah == 0.0f)))
     return ((double)j + 0.5 * (double)F) / (double)rho;
-  float q0 = __fmul_rn(h, rc);
-  q0 = __fmaf_rn(__fmaf_rn(-q0, rho, h), rc, q0);
-  const float r0 = __fmaf_rn(-q0, rho, h);
+  float q0 = __fmul_rn(h, rc2);
+  q0 = __fmaf_rn(__fmaf_rn(-q0, r2, h), rc2, q0);
+  const float r0 = __fmaf_rn(-q0, r2, h);
   const float e0 = __fadd_rn(r0, l), eb = __fsub_rn(e0, r0);
   const float e1 = __fadd_rn(__fsub_rn(r0, __fsub_rn(e0, eb)), __fsub_rn(l, eb));
-  const float q1 = __fmul_rn(e0, rc);
-  const float q2 = __fmul_rn(__fadd_rn(__fmaf_rn(-q1, rho, e0), e1), rc);
+  const float q1 = __fmul_rn(e0, rc2);
+  const float q2 = __fmul_rn(__fadd_rn(__fmaf_rn(-q1, r2, e0), e1), rc2);
   return f64_from_f32(q0) + (f64_from_f32(q1) + f64_from_f32(q2));
 }
 

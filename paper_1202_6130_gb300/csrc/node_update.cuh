@@ -50,9 +50,9 @@ __device__ __forceinline__ void write_moments(const Args& a, int64_t n, T rho, T
     a.out_ux[n] = (double)jx + 0.5 * (double)Fx;
     a.out_uy[n] = (double)jy + 0.5 * (double)Fy;
   } else if constexpr (sizeof(T) == 4) {
-    const float rc = __frcp_rn(rho);
-    a.out_ux[n] = half_force_velocity(jx, Fx, rho, rc);
-    a.out_uy[n] = half_force_velocity(jy, Fy, rho, rc);
+    const float r2 = __fadd_rn(rho, rho), rc2 = __frcp_rn(r2);
+    a.out_ux[n] = half_force_velocity(jx, Fx, rho, r2, rc2);
+    a.out_uy[n] = half_force_velocity(jy, Fy, rho, r2, rc2);
   } else {
     const T y = T(1) / rho;
     a.out_ux[n] = div_rho<T>(jx + 0.5 * Fx, rho, y);
